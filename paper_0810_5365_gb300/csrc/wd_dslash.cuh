@@ -17,6 +17,7 @@
 #include <map>
 #include <type_traits>
 
+#include "wd_fix64.cuh"
 #include "wd_internal.h"
 
 namespace wd {
@@ -543,6 +544,105 @@ __device__ __forceinline__ float hops_f16(__half2 (&ah)[12], const void* __restr
   return smax;
 }
 
+// The eight neighbours of a site (checkerboard indices of the other parity,
+// hop order f0 b0 f1 b1 f2 b2 f3 b3) and its time-boundary flags.
+struct Nbrs {
+  int n[8];
+  bool fflip, bflip;  // the forward / backward time hop crosses the boundary
+  bool funit, bunit;  // the forward / backward time link is the identity
+};
+
+// The eight hops of one site in the site's working precision.
+template <int P, int RC, bool DAG, typename R, bool COH>
+__device__ __forceinline__ void hops_chain(cx<R> (&acc)[12], const void* __restrict__ in,
+                                           const void* __restrict__ ga, int p, int cb,
+                                           const Nbrs& nb, int VP) {
+  constexpr int SF = DAG ? -1 : 1;
+  constexpr int SB_ = -SF;
+  const int q = 1 - p;
+#pragma unroll
+  for (int k = 0; k < 12; k++) acc[k] = mk<R>(0, 0);
+  hop<P, RC, 0, SF, true, R, COH>(acc, in, ga, nb.n[0], 0 + p, cb, false, VP);
+  hop<P, RC, 0, SB_, false, R, COH>(acc, in, ga, nb.n[1], 0 + q, nb.n[1], false, VP);
+  hop<P, RC, 1, SF, true, R, COH>(acc, in, ga, nb.n[2], 2 + p, cb, false, VP);
+  hop<P, RC, 1, SB_, false, R, COH>(acc, in, ga, nb.n[3], 2 + q, nb.n[3], false, VP);
+  hop<P, RC, 2, SF, true, R, COH>(acc, in, ga, nb.n[4], 4 + p, cb, false, VP);
+  hop<P, RC, 2, SB_, false, R, COH>(acc, in, ga, nb.n[5], 4 + q, nb.n[5], false, VP);
+  hop<P, RC, 3, SF, true, R, COH>(acc, in, ga, nb.n[6], 6 + p, cb, nb.fflip, VP, nb.funit);
+  hop<P, RC, 3, SB_, false, R, COH>(acc, in, ga, nb.n[7], 6 + q, nb.n[7], nb.bflip, VP, nb.bunit);
+}
+
+// ... for the FP64 sites whose values do not fit the fixed-point sum
+template <int RC, bool DAG, bool COH>
+__device__ __noinline__ void hops_chain_f64(cx<double> (&acc)[12], const void* __restrict__ in,
+                                            const void* __restrict__ ga, int p, int cb,
+                                            const Nbrs& nb, int VP) {
+  hops_chain<WD_F64, RC, DAG, double, COH>(acc, in, ga, p, cb, nb, VP);
+}
+
+// One FP64 hop into the fixed-point sums (wd_fix64.cuh).
+template <int RC, int S, bool FWD, bool COH>
+__device__ __forceinline__ void hop_fix(FixSite& fx, int mu, const void* __restrict__ in,
+                                        const void* __restrict__ gauge, int nb, int region,
+                                        int lcb, bool flip, int VP, bool unit) {
+  cx<double> psi[12], h[6];
+  load_spinor<WD_F64, double, COH>(psi, in, nb, VP);
+  double u[RC];
+  if (unit) {
+#pragma unroll
+    for (int k = 0; k < RC; k++) u[k] = 0.0;
+  } else {
+    constexpr int NC = RC / 2;
+    const double2* g = (const double2*)gauge + (size_t)region * VP * NC;
+#pragma unroll
+    for (int k = 0; k < NC; k++) {
+      const double2 v = __ldg(g + sbi(lcb, k, NC));
+      u[2 * k] = v.x;
+      u[2 * k + 1] = v.y;
+    }
+  }
+  switch (mu) {
+    case 0: project<0, S>(psi, h); break;
+    case 1: project<1, S>(psi, h); break;
+    case 2: project<2, S>(psi, h); break;
+    default: project<3, S>(psi, h); break;
+  }
+  fix_hop<S, FWD, RC>(fx, mu, h, u, flip, unit);
+}
+
+// The eight hops of one FP64 site: fixed point, or the FP64 chain where the
+// values do not fit it.  24^3x48, one parity, us per launch: FP64 chain 541
+// (recon 18) and 788 (recon 12, which rebuilds row 2 on the FP64 pipe), fixed
+// point 175 and 196.  What bounds it now: the integer pipes (ALU 42 % busy)
+// through the latency of dependent instructions, with 12 warps per SM at 168
+// registers; 8 or 16 warps (255 registers, or 128 and spills) are slower.  The
+// directions are a loop, not unrolled: eight copies of the hop (200 KB of
+// code) ran out of the instruction cache and took 500 us.
+template <int RC, bool DAG, bool COH>
+__device__ __forceinline__ void hops_f64(cx<double> (&acc)[12], const void* __restrict__ in,
+                                         const void* __restrict__ ga, int p, int cb,
+                                         const Nbrs& nb, int VP) {
+  constexpr int SF = DAG ? -1 : 1;
+  FixSite fx;
+  fix_begin(fx);
+#pragma unroll 1
+  for (int mu = 0; mu < 4; mu++) {
+    const int f = mu == 0 ? nb.n[0] : mu == 1 ? nb.n[2] : mu == 2 ? nb.n[4] : nb.n[6];
+    const int b = mu == 0 ? nb.n[1] : mu == 1 ? nb.n[3] : mu == 2 ? nb.n[5] : nb.n[7];
+    hop_fix<RC, SF, true, COH>(fx, mu, in, ga, f, 2 * mu + p, cb, mu == 3 && nb.fflip, VP,
+                               mu == 3 && nb.funit);
+    hop_fix<RC, -SF, false, COH>(fx, mu, in, ga, b, 2 * mu + 1 - p, b, mu == 3 && nb.bflip, VP,
+                                 mu == 3 && nb.bunit);
+  }
+  if (fix_ok(fx)) {
+#pragma unroll
+    for (int k = 0; k < 12; k++)
+      acc[k] = mk<double>(fix_double(fx.r[k], fx.E), fix_double(fx.i[k], fx.E));
+  } else {
+    hops_chain_f64<RC, DAG, COH>(acc, in, ga, p, cb, nb, VP);
+  }
+}
+
 // TG: links in temporal gauge (compile-time, so that the ordinary kernel keeps
 // its register budget)
 // BS sites per CTA; the register budget per thread is that of the 128-site
@@ -585,18 +685,15 @@ __global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>
     const bool funit = TG && !fflip;
     const bool bunit = TG && !bflip;
 
-    // forward hops use (1 - s gamma), backward (1 + s gamma)
-    constexpr int SF = DAG ? -1 : 1;
-    constexpr int SB_ = -SF;
-    const int q = 1 - p;
     const int VP = g.Vh_pad;
 
     cx<R> acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; k++) acc[k] = mk<R>(0, 0);
 
     bool stored = false;
     if constexpr (P == WD_F16) {
+      // forward hops use (1 - s gamma), backward (1 + s gamma)
+      constexpr int SF = DAG ? -1 : 1;
+      constexpr int SB_ = -SF;
       __half2 ah[12];
       const float kf = (float)a.a * hops_f16<SF, SB_>(ah, a.in, a.gauge, p, cb, f0, b0, f1, b1,
                                                       f2, b2, f3, b3, fflip, bflip, funit, bunit,
@@ -608,14 +705,11 @@ __global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>
         f16_widen(acc, ah, kf);
       }
     } else {
-      hop<P, RC, 0, SF, true>(acc, a.in, a.gauge, f0, 0 + p, cb, false, VP);
-      hop<P, RC, 0, SB_, false>(acc, a.in, a.gauge, b0, 0 + q, b0, false, VP);
-      hop<P, RC, 1, SF, true>(acc, a.in, a.gauge, f1, 2 + p, cb, false, VP);
-      hop<P, RC, 1, SB_, false>(acc, a.in, a.gauge, b1, 2 + q, b1, false, VP);
-      hop<P, RC, 2, SF, true>(acc, a.in, a.gauge, f2, 4 + p, cb, false, VP);
-      hop<P, RC, 2, SB_, false>(acc, a.in, a.gauge, b2, 4 + q, b2, false, VP);
-      hop<P, RC, 3, SF, true>(acc, a.in, a.gauge, f3, 6 + p, cb, fflip, VP, funit);
-      hop<P, RC, 3, SB_, false>(acc, a.in, a.gauge, b3, 6 + q, b3, bflip, VP, bunit);
+      const Nbrs nb = {{f0, b0, f1, b1, f2, b2, f3, b3}, fflip, bflip, funit, bunit};
+      if constexpr (P == WD_F64)
+        hops_f64<RC, DAG, false>(acc, a.in, a.gauge, p, cb, nb, VP);
+      else
+        hops_chain<P, RC, DAG, R, false>(acc, a.in, a.gauge, p, cb, nb, VP);
     }
 
     if constexpr (P != WD_F16) {  // (the FP16 hops apply a themselves)

@@ -1,0 +1,338 @@
+// The FP64 hopping sum in 64-bit fixed point on the integer pipe.
+//
+// GB300 issues FP64 at 1/64 of its FP32 rate (1.7 DADD lanes per SM and clock
+// measured) but 64 lanes of 32 x 32 + 64 bit multiply-adds (mad.wide.s32) or
+// 64-bit adds.  A hop needs 36 FP64 additions and 72 multiply-adds, so the
+// FP64 pipe bounds the FP64 kernel at about 500 clocks per site and SM, seven
+// times its memory time.  Here only the 12 additions of the spin projection
+// stay on that pipe; the SU(3) product and the sum over the eight hops run on
+// integers.
+//
+// Formats (E: the site's scale, a biased exponent not below that of any
+// projected component seen so far, e = E - 1023):
+//   half spinor  h = H 2^(e-60), |H| < 2^61
+//   link         u = V 2^-59,    |V| < 2^59 (1 + 2^-20)
+//   sums         t = T 2^(e-55), below 2^62 after eight hops
+// H and V are cut into two signed 32-bit limbs, x = x.h 2^32 + x.l, and
+// H V = H.h V.h 2^64 + (H.h V.l + H.l V.h) 2^32 + H.l V.l.  The last product
+// is dropped (below 2^-56 of the largest |h|, rms), the middle ones are summed
+// and rounded once per component and hop.  The FP64 chain rounds each of
+// its 6 + 1 additions per hop at 2^-53 of the partial sum.  Errors relative to
+// the rms component of the site, both against 64-bit-mantissa references:
+// fixed point 0.58e-16, chain 1.42e-16 on Gaussian neighbours of one size; the
+// fixed-point one is the smaller for every form tried (unit links, single
+// colours, sizes spread over 2^+-40: tests/host/fix64_check.cu).
+//
+// A site falls back to the FP64 chain when a value does not fit: |u| above 1
+// or a link that is small throughout (not SU(3)), infinities, NaN, or
+// exponents near the ends of the range.
+//
+// Instructions per hop: 30 conversions of 11 (a 64-bit shift written on two
+// 32-bit words: on a 64-bit variable the compiler took 16), 216 multiply-adds,
+// about 100 for the sums and 60 for the scale.
+#pragma once
+
+#include <string.h>
+
+#include "wd_common.cuh"
+
+namespace wd {
+
+struct Limb {
+  int h, l;
+};
+
+// 64-bit accumulators of a site: the four spins of the output, as T above
+struct FixSite {
+  long long r[12], i[12];
+  int E;          // biased exponent of the scale
+  unsigned any;   // non-zero: some neighbour was not zero
+  unsigned bad;   // non-zero: a value did not fit
+};
+
+constexpr int FIX_EMIN = 128;   // smallest and largest scale handled
+constexpr int FIX_EMAX = 1980;
+constexpr unsigned FIX_UMAX = 0x3ff00000u;  // high words of |u| < 1 + 2^-20 ...
+constexpr unsigned FIX_UMIN = 0x3fc00000u;  // ... and of 1/8 (an SU(3) row has a real >= 0.23)
+
+__host__ __device__ __forceinline__ unsigned long long d_bits(double x) {
+  unsigned long long b;
+  memcpy(&b, &x, 8);
+  return b;
+}
+
+// (hi : lo) >> s, 0 for s > 63
+__host__ __device__ __forceinline__ void shr_pair(unsigned& hi, unsigned& lo, int s) {
+#ifdef __CUDA_ARCH__
+  asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %0};\n\tshr.u64 t, t, %2;\n\tmov.b64 {%1, %0}, t;\n\t}"
+      : "+r"(hi), "+r"(lo) : "r"(s));
+#else
+  const unsigned long long v = s > 63 ? 0 : (((unsigned long long)hi << 32) | lo) >> s;
+  hi = (unsigned)(v >> 32);
+  lo = (unsigned)v;
+#endif
+}
+
+__host__ __device__ __forceinline__ Limb fix_split(long long v) {
+  Limb o;
+  o.l = (int)(unsigned)v;
+  o.h = (int)(v >> 32) + (int)((unsigned)o.l >> 31);
+  return o;
+}
+
+// |x| with its leading bit (of 2^e) at bit 63 - (s - e), truncated, with x's
+// sign; a negative value comes out one unit low (x ^ -1 for -x), as
+// fix_neg's do
+__host__ __device__ __forceinline__ Limb fix_limbs(unsigned long long b, int s) {
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned a = hi & 0x7fffffffu;
+  const int sh = s - (int)(a >> 20);
+  unsigned top = ((a << 11) | (lo >> 21)) | 0x80000000u, bot = lo << 11;
+  shr_pair(top, bot, sh);
+  const unsigned m = (unsigned)((int)hi >> 31);
+  Limb o;
+  o.l = (int)(bot ^ m);
+  o.h = (int)(top ^ m) + (int)((unsigned)o.l >> 31);
+  return o;
+}
+
+__host__ __device__ __forceinline__ Limb fix_neg(Limb a) {
+  Limb o;
+  o.h = -a.h;
+  o.l = ~a.l;
+  return o;
+}
+
+// one real of a sum of products
+struct FixAcc {
+  long long A, B;
+};
+__host__ __device__ __forceinline__ void fix_mac(FixAcc& s, Limb u, Limb h) {
+  s.A += (long long)u.h * h.h;
+  s.B += (long long)u.h * h.l;
+  s.B += (long long)u.l * h.h;
+}
+__host__ __device__ __forceinline__ long long fix_round(const FixAcc& s) {
+  return s.A + (s.B >> 32);
+}
+
+// conj(a b - c d) as a link element (row 2 of an SU(3) matrix)
+__host__ __device__ __forceinline__ void fix_cross(Limb (&o)[2], const Limb (&a)[2],
+                                                   const Limb (&b)[2], const Limb (&c)[2],
+                                                   const Limb (&d)[2]) {
+  const Limb nbi = fix_neg(b[1]), ndr = fix_neg(d[0]), nbr = fix_neg(b[0]);
+  FixAcc re = {0, 1LL << 26}, im = {0, 1LL << 26};
+  fix_mac(re, a[0], b[0]);
+  fix_mac(re, a[1], nbi);
+  fix_mac(re, c[0], ndr);
+  fix_mac(re, c[1], d[1]);
+  // -(a.r b.i + a.i b.r - c.r d.i - c.i d.r)
+  fix_mac(im, a[0], nbi);
+  fix_mac(im, a[1], nbr);
+  fix_mac(im, c[0], d[1]);
+  fix_mac(im, c[1], d[0]);
+  // products 2^-118 -> 2^-59
+  o[0] = fix_split(re.A * 32 + (re.B >> 27));
+  o[1] = fix_split(im.A * 32 + (im.B >> 27));
+}
+
+// Site state before its first hop.
+__host__ __device__ __forceinline__ void fix_begin(FixSite& acc) {
+#pragma unroll
+  for (int k = 0; k < 12; k++) acc.r[k] = acc.i[k] = 0;
+  acc.E = FIX_EMIN;
+  acc.any = acc.bad = 0;
+}
+
+// Raise the site's scale to that of the projected half spinor h when h is
+// larger (to one bit above it, so that few of the later hops raise it again:
+// each time costs the shift of all sums).  False: h vanishes, nothing to add.
+__host__ __device__ __forceinline__ bool fix_scale(FixSite& acc, const cx<double> (&h)[6]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    const unsigned a = (unsigned)(d_bits(h[k].r) >> 32) & 0x7fffffffu;
+    const unsigned b = (unsigned)(d_bits(h[k].i) >> 32) & 0x7fffffffu;
+    m = m > a ? m : a;
+    m = m > b ? m : b;
+  }
+  acc.any |= m;
+  if (m == 0) {
+    // a zero neighbour (point sources), or denormals of up to 2^-1043
+    unsigned long long lows = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) lows |= d_bits(h[k].r) | d_bits(h[k].i);
+    acc.bad |= (unsigned)lows;
+    return false;
+  }
+  const int e = (int)(m >> 20);
+  if (e > acc.E) {
+    const int d = e + 1 - acc.E < 63 ? e + 1 - acc.E : 63;
+    acc.E = e + 1;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      acc.r[k] >>= d;
+      acc.i[k] >>= d;
+    }
+  }
+  return true;
+}
+
+// The largest |high word| of n link reals so far, and at the end whether the
+// link is one that V can hold.
+__host__ __device__ __forceinline__ void fix_link_max(unsigned& um, unsigned long long b) {
+  const unsigned a = (unsigned)(b >> 32) & 0x7fffffffu;
+  um = um > a ? um : a;
+}
+
+// t = (row c of U h) or (row c of U^+ h) for one of the two half spinors:
+// v[d] = U[c][d] or U[d][c], H[d] the limbs of h
+template <bool FWD>
+__host__ __device__ __forceinline__ void fix_row(long long& tr, long long& ti,
+                                                 const Limb (&v)[3][2], const Limb (*H)[2]) {
+  FixAcc re = {0, 1LL << 31}, im = {0, 1LL << 31};
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const Limb n = fix_neg(H[d][FWD ? 1 : 0]);
+    fix_mac(re, v[d][0], H[d][0]);
+    fix_mac(re, v[d][1], FWD ? n : H[d][1]);
+    fix_mac(im, v[d][0], H[d][1]);
+    fix_mac(im, v[d][1], FWD ? H[d][0] : n);
+  }
+  tr = fix_round(re);
+  ti = fix_round(im);
+}
+
+// Colour c of the expansion of expand_add: upper spins t0, t1, lower spins
+// +-S t or +-S i t (of direction mu).
+template <int S>
+__host__ __device__ __forceinline__ void fix_expand(FixSite& acc, int mu, int c, long long r0,
+                                                    long long i0, long long r1, long long i1) {
+  acc.r[c] += r0;
+  acc.i[c] += i0;
+  acc.r[3 + c] += r1;
+  acc.i[3 + c] += i1;
+  auto add = [&](int k, long long r, long long i, int sgn) {
+    acc.r[k] = sgn > 0 ? acc.r[k] + r : acc.r[k] - r;
+    acc.i[k] = sgn > 0 ? acc.i[k] + i : acc.i[k] - i;
+  };
+  // sgn * i t = (-sgn t.i, sgn t.r)
+  auto add_i = [&](int k, long long r, long long i, int sgn) {
+    acc.r[k] = sgn > 0 ? acc.r[k] - i : acc.r[k] + i;
+    acc.i[k] = sgn > 0 ? acc.i[k] + r : acc.i[k] - r;
+  };
+  switch (mu) {
+    case 0:  // lower = (-S i t1, -S i t0)
+      add_i(6 + c, r1, i1, -S);
+      add_i(9 + c, r0, i0, -S);
+      break;
+    case 1:  // lower = (-S t1, S t0)
+      add(6 + c, r1, i1, -S);
+      add(9 + c, r0, i0, S);
+      break;
+    case 2:  // lower = (-S i t0, S i t1)
+      add_i(6 + c, r0, i0, -S);
+      add_i(9 + c, r1, i1, S);
+      break;
+    default:  // lower = (-S t0, -S t1)
+      add(6 + c, r0, i0, -S);
+      add(9 + c, r1, i1, -S);
+      break;
+  }
+}
+
+// One hop of direction mu: the projected half spinor h (six complex doubles)
+// times the link u (RC reals as stored; not read when unit), added to the
+// site's sums.  Colour by colour, so that only one row of products is live
+// beside the sums.
+template <int S, bool FWD, int RC>
+__host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<double> (&h)[6],
+                                                 const double (&u)[RC], bool flip, bool unit) {
+  if (!fix_scale(acc, h)) return;
+  Limb H[6][2];
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    H[k][0] = fix_limbs(d_bits(h[k].r), acc.E + 3);
+    H[k][1] = fix_limbs(d_bits(h[k].i), acc.E + 3);
+  }
+  if (flip) {
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      H[k][0] = fix_neg(H[k][0]);
+      H[k][1] = fix_neg(H[k][1]);
+    }
+  }
+  if (unit) {
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      auto t = [](Limb a) { return ((((long long)a.h << 32) + a.l) + 16) >> 5; };
+      fix_expand<S>(acc, mu, c, t(H[c][0]), t(H[c][1]), t(H[3 + c][0]), t(H[3 + c][1]));
+    }
+    return;
+  }
+  Limb U[9][2];
+  unsigned um = 0;
+  if (RC == 12) {
+#pragma unroll
+    for (int k = 0; k < RC; k++) {
+      fix_link_max(um, d_bits(u[k]));
+      U[k >> 1][k & 1] = fix_limbs(d_bits(u[k]), 1023 + 4);
+    }
+    fix_cross(U[6], U[1], U[5], U[2], U[4]);
+    fix_cross(U[7], U[2], U[3], U[0], U[5]);
+    fix_cross(U[8], U[0], U[4], U[1], U[3]);
+    // (rows that are not orthonormal can give a larger row 2)
+    unsigned big = 0;
+#pragma unroll
+    for (int k = 6; k < 9; k++)
+      big |= ((unsigned)(U[k][0].h + (1 << 27) + 128) | (unsigned)(U[k][1].h + (1 << 27) + 128));
+    acc.bad |= big >> 29;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    Limb v[3][2];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const int k = FWD ? c * 3 + d : d * 3 + c;
+        if (RC == 12) {
+          v[d][j] = U[k][j];
+        } else {
+          fix_link_max(um, d_bits(u[2 * k + j]));
+          v[d][j] = fix_limbs(d_bits(u[2 * k + j]), 1023 + 4);
+        }
+      }
+    }
+    long long r0, i0, r1, i1;
+    fix_row<FWD>(r0, i0, v, &H[0]);
+    fix_row<FWD>(r1, i1, v, &H[3]);
+    fix_expand<S>(acc, mu, c, r0, i0, r1, i1);
+  }
+  acc.bad |= (um > FIX_UMAX || um < FIX_UMIN) ? 1u : 0u;
+}
+
+// whether the site's sums are valid (else: the FP64 chain)
+__host__ __device__ __forceinline__ bool fix_ok(const FixSite& a) {
+  return a.bad == 0 && a.E < FIX_EMAX && (a.E > FIX_EMIN || a.any == 0);
+}
+
+// T 2^(E - 1023 - 55) as a double, rounded to nearest
+__host__ __device__ __forceinline__ double fix_double(long long t, int E) {
+  const long long s = t >> 63;
+  const unsigned long long m = (unsigned long long)((t ^ s) - s);
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)m);
+#else
+  const int lz = m ? __builtin_clzll(m) : 64;
+#endif
+  const unsigned long long n = m << (lz & 63);
+  unsigned long long b = ((unsigned long long)(E + 7 - lz) << 52) + (n >> 11) + ((n >> 10) & 1);
+  b |= (unsigned long long)s & 0x8000000000000000ull;
+  if (m == 0) b = 0;
+  double d;
+  memcpy(&d, &b, 8);
+  return d;
+}
+
+}  // namespace wd

@@ -79,10 +79,8 @@ struct MrhsMinBlocks {
 template <int P, int RC, bool DAG, bool NORM, bool COH = false>
 __device__ __forceinline__ real_of<P> mrhs_site(const MrhsProblem& pr, int cb, int r) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
-  constexpr int SF = DAG ? -1 : 1;
-  constexpr int SB_ = -SF;
   const Geom& g = pr.g;
-  const int p = pr.parity, qq = 1 - p, VP = g.Vh_pad;
+  const int p = pr.parity, VP = g.Vh_pad;
   int x0, x1, x2, x3;
   cb_coords(cb, p, g, x0, x1, x2, x3);
   const int row = cb - (x0 >> 1);
@@ -99,11 +97,11 @@ __device__ __forceinline__ real_of<P> mrhs_site(const MrhsProblem& pr, int cb, i
   const void* in = (const char*)pr.in + (size_t)r * pr.s_in;
   const void* ga = pr.gauge;
   cx<R> acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; k++) acc[k] = mk<R>(0, 0);
   void* out = (char*)pr.out + (size_t)r * pr.s_out;
   bool stored = false;
   if constexpr (P == WD_F16) {
+    constexpr int SF = DAG ? -1 : 1;
+    constexpr int SB_ = -SF;
     __half2 ah[12];
     const float kf = (float)pr.a * hops_f16<SF, SB_, COH>(ah, in, ga, p, cb, f0, b0, f1, b1, f2,
                                                          b2, f3, b3, fflip, bflip, false, false,
@@ -115,14 +113,11 @@ __device__ __forceinline__ real_of<P> mrhs_site(const MrhsProblem& pr, int cb, i
       f16_widen(acc, ah, kf);
     }
   } else {
-    hop<P, RC, 0, SF, true, R, COH>(acc, in, ga, f0, 0 + p, cb, false, VP);
-    hop<P, RC, 0, SB_, false, R, COH>(acc, in, ga, b0, 0 + qq, b0, false, VP);
-    hop<P, RC, 1, SF, true, R, COH>(acc, in, ga, f1, 2 + p, cb, false, VP);
-    hop<P, RC, 1, SB_, false, R, COH>(acc, in, ga, b1, 2 + qq, b1, false, VP);
-    hop<P, RC, 2, SF, true, R, COH>(acc, in, ga, f2, 4 + p, cb, false, VP);
-    hop<P, RC, 2, SB_, false, R, COH>(acc, in, ga, b2, 4 + qq, b2, false, VP);
-    hop<P, RC, 3, SF, true, R, COH>(acc, in, ga, f3, 6 + p, cb, fflip, VP);
-    hop<P, RC, 3, SB_, false, R, COH>(acc, in, ga, b3, 6 + qq, b3, bflip, VP);
+    const Nbrs nb = {{f0, b0, f1, b1, f2, b2, f3, b3}, fflip, bflip, false, false};
+    if constexpr (P == WD_F64)
+      hops_f64<RC, DAG, COH>(acc, in, ga, p, cb, nb, VP);
+    else
+      hops_chain<P, RC, DAG, R, COH>(acc, in, ga, p, cb, nb, VP);
   }
   if constexpr (P != WD_F16) {  // (the FP16 hops apply a themselves)
     const R ca = (R)pr.a;
