@@ -116,8 +116,9 @@ const char *wd_error_string(int status);
 /* cudaError_t of the last failed CUDA call (0 if none). */
 int wd_last_cuda_error(void);
 
-/* Free the library's cached workspace (solver fields, reduction scratch,
- * captured graphs).  Caller buffers are untouched.  Safe to call twice. */
+/* Free the library's cached workspace (solver fields, reduction scratch, the
+ * network calls' scratch of at most 1 GiB, captured graphs).  Caller buffers
+ * are untouched.  Safe to call twice. */
 void wd_finalize(void);
 
 /* ------------------------------------------------------------------ */

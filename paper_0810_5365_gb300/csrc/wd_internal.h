@@ -134,6 +134,10 @@ struct State {
   size_t partials_cap = 0;  // doubles
   int num_sms = 0;
   int* dev_flag = nullptr;  // device int: set by kernels whose bounded waits gave up
+  // fields between the layers of wd_nn_apply*, partials of wd_nn_wgrad
+  void* nn_scratch = nullptr;
+  size_t nn_scratch_bytes = 0;
+  int nn_scratch_dev = -1;
   // polls of the first bounded wait of the asynchronous kernels (wd_set_wait_limit)
   long wait_limit = 1L << 22;
 };
