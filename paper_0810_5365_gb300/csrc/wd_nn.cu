@@ -138,40 +138,83 @@ static cudaError_t nn_layer(int cin, int cout, const Geom& g, const void* gauge,
 // sums them in CTA order)
 // ---------------------------------------------------------------------------
 
-// out[j] (+)= sum_t partials[t][j], t in order
-__global__ void nn_sum_tiles(const float* __restrict__ partials, int ntiles, int n, float* out,
-                             int accumulate) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+// out[j] (+)= sum_t partials[t][j] in FP64, in a fixed order: slice y of a
+// block adds t = y, y + NN_SUM_SLICES, ..., then the slices are added in
+// order.  One thread per j walked up to 304 partials one L2 load after another
+// (28 us for 1152 sums); 16 slices of at most 19 take 7.8 us.
+constexpr int NN_SUM_SLICES = 16;
+
+__global__ void __launch_bounds__(32 * NN_SUM_SLICES)
+    nn_sum_tiles(const float* __restrict__ partials, int ntiles, int n, float* out,
+                 int accumulate) {
+  __shared__ double sm[NN_SUM_SLICES][32];
+  const int j = blockIdx.x * 32 + threadIdx.x;
   double s = 0.0;
-  for (int t = 0; t < ntiles; t++) s += (double)partials[(size_t)t * n + j];
-  out[j] = accumulate ? out[j] + (float)s : (float)s;
+  if (j < n) {
+#pragma unroll 4
+    for (int t = threadIdx.y; t < ntiles; t += NN_SUM_SLICES)
+      s += (double)partials[(size_t)t * n + j];
+  }
+  sm[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && j < n) {
+#pragma unroll
+    for (int y = 1; y < NN_SUM_SLICES; y++) s += sm[y][threadIdx.x];
+    out[j] = accumulate ? out[j] + (float)s : (float)s;
+  }
 }
 
 // ---------------------------------------------------------------------------
 // weight gradient on the tensor cores: for all nine directions at once,
 //   G^T[d C_in + i][2o + part] = sum_{x, a} (T_d phi)[i][a] x delta-row,
 // with the real form of the complex product conj-contracted over (site,
-// colour): the A rows are the transported input channels [t_r | t_i] (9 C_in
-// of the M = 128 rows, the rest zero), the B rows are [delta_r | delta_i] for
-// Re G and [delta_i | -delta_r] for Im G (2 C_out of N = 16 rows).  K runs over
-// (part, colour, site) of 32-site blocks: 192 = 12 chunks of 16 per block.
-// Each persistent CTA accumulates its blocks in TMEM (FP32), writes its
-// partial gradient, and the partials are summed over CTAs in a fixed order.
+// colour): the A rows are the transported input channels (9 C_in of the M =
+// 128 rows, the rest zero), the B rows are [delta_r, delta_i] for Re G and
+// [delta_i, -delta_r] for Im G (2 C_out of N = 16 rows).  K runs over (site,
+// colour, part) of 32-site blocks: 192 = 12 chunks of 16 per block, part
+// innermost, so that each complex value is one 4-byte store and the 32 sites
+// of a warp fill consecutive words.  Each persistent CTA accumulates its blocks
+// in TMEM (FP32), writes its partial gradient, and the partials are summed
+// over CTAs in a fixed order.
+//
+// One warp per direction (nine, both channel halves with one link load).
+// What bounds it: the loads of a block (24 + 12 + 6 16-byte words per site and
+// direction) before its barrier, with 18 warps per SM (issue slots 51 % busy).
+// Eight warps sharing the nine directions (three rounds where 2.25 were
+// needed), each half with its own link load, and 2-byte stores into 4 banks
+// took, us on 16^3x32 / 32^3x64 (this kernel in brackets): 8 -> 8 70.5 / 1187
+// [57 / 879], 8 -> 4 66 / 1143 [50 / 793], 4 -> 8 50 / 901 [39 / 622].
 // ---------------------------------------------------------------------------
 
 constexpr int WG_SITES = 32;                    // sites per K block
 constexpr int WG_KCH = 2 * 3 * WG_SITES / 16;   // K chunks of 16 per block
-constexpr uint32_t WG_ACH = 128 * 16 * 2;       // one A chunk (M = 128 rows), bytes
-constexpr uint32_t WG_BCH = 16 * 16 * 2;        // one B chunk (N = 16 rows), bytes
+// Operand layout (K-major, no swizzle): core matrices of 8 rows x 16 bytes,
+// 128 bytes apart along the rows (SBO); the two of a chunk along K are LBO
+// apart, and the chunks ACH / BCH.  LBO is 16 and the chunk stride 32 bytes
+// above a multiple of 128, so that word w of a row (w = 3 site + colour) lies
+// in bank w mod 32 (plus the row's offset): the stores of a warp, at every
+// third word, are free of conflicts.
+constexpr uint32_t WG_SBO = 128;
+constexpr uint32_t WG_ALBO = 128 * 16 + 16;     // M = 128 rows
+constexpr uint32_t WG_ACH = 2 * 128 * 16 + 32;
+constexpr uint32_t WG_BLBO = 16 * 16 + 16;      // N = 16 rows
+constexpr uint32_t WG_BCH = 2 * 16 * 16 + 32;
 constexpr uint32_t WG_BUF = WG_KCH * (WG_ACH + WG_BCH);
-constexpr int WG_THREADS = 256;
+constexpr int WG_THREADS = 32 * NN_NDIR;
+
+// byte offset of word w of row 0, and of row r
+__device__ __forceinline__ uint32_t wg_word(int w, uint32_t ch, uint32_t lbo) {
+  return (uint32_t)(w >> 3) * ch + (uint32_t)((w >> 2) & 1) * lbo + (uint32_t)(w & 3) * 4;
+}
+__device__ __forceinline__ uint32_t wg_row(int r) {
+  return (uint32_t)(r >> 3) * WG_SBO + (uint32_t)(r & 7) * 16;
+}
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(WG_THREADS) nn_wgrad_tc_kernel(const NnLayerArgs A,
-                                                                 const char* __restrict__ delta,
-                                                                 size_t delta_half, int nblocks,
-                                                                 float* partials) {
+__global__ void __launch_bounds__(WG_THREADS, 2) nn_wgrad_tc_kernel(const NnLayerArgs A,
+                                                                    const char* __restrict__ delta,
+                                                                    size_t delta_half, int nblocks,
+                                                                    float* partials) {
   extern __shared__ __align__(128) unsigned char wg_smem[];  // 2 buffers of WG_BUF
   __shared__ uint64_t bar[2];
   __shared__ uint32_t tmem_base;
@@ -196,13 +239,13 @@ __global__ void __launch_bounds__(WG_THREADS) nn_wgrad_tc_kernel(const NnLayerAr
   const uint32_t tbase = tmem_base;
   const uint32_t idesc = make_idesc_bf16(128, 16);
   const int bpp = (g.Vh + WG_SITES - 1) / WG_SITES;  // blocks per parity
-  // work split of the 8 warps: CIN = 8: warps w and w + 4 transport channels
-  // 0-3 and 4-7 of directions w, w + 4, w + 8; CIN = 4: warps 0-3 transport
-  // directions w, w + 4, w + 8 and warps 4-7 stage the delta rows
-  constexpr bool SPLIT = CIN == 8;
-  const int dw = warp & 3;
-  const int c0 = SPLIT ? 4 * (warp >> 2) : 0;
-  const bool transports = SPLIT || warp < 4;
+  const int d = warp;  // one direction per warp
+  uint32_t wa[3], wb[3];  // this site's words (one per colour) in an A and a B row
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    wa[a] = wg_word(3 * lane + a, WG_ACH, WG_ALBO);
+    wb[a] = wg_word(3 * lane + a, WG_BCH, WG_BLBO);
+  }
   bool ok = true;
   uint32_t G = 0;  // blocks issued by this CTA
 
@@ -214,81 +257,70 @@ __global__ void __launch_bounds__(WG_THREADS) nn_wgrad_tc_kernel(const NnLayerAr
     const int p = blk / bpp;
     const int cb = (blk - p * bpp) * WG_SITES + lane;
     const bool valid = cb < g.Vh;
-    if (transports) {
+    int n = cb, x3 = 0;
+    if (valid) {
       int nb[NN_NDIR];
-      int x3 = 0;
-      if (valid) nn_nbr(nb, x3, cb, p, g);
-      for (int d = dw; d < NN_NDIR; d += 4) {
-        cx<float> t[12];
-        if (valid) {
-          nn_transport4<CIN>(t, A, d, p, cb, nb[d], x3, c0);
-        } else {
+      nn_nbr(nb, x3, cb, p, g);
 #pragma unroll
-          for (int k = 0; k < 12; k++) t[k] = mk<float>(0.f, 0.f);
+      for (int k = 1; k < NN_NDIR; k++) n = d == k ? nb[k] : n;
+    }
+    cx<float> u[9];
+    float sg = 1.f;
+    if (valid && d > 0) sg = nn_link(u, A, d, p, cb, n, x3);
+    const char* src = A.in + (d == 0 ? p : 1 - p) * A.in_half;
+#pragma unroll
+    for (int c0 = 0; c0 < CIN; c0 += 4) {
+      cx<float> t[12];
+      if (!valid) {
+#pragma unroll
+        for (int k = 0; k < 12; k++) t[k] = mk<float>(0.f, 0.f);
+      } else if (d == 0) {
+        nn_load4<CIN>(t, src, cb, c0);
+      } else {
+        cx<float> v[12];
+        nn_load4<CIN>(v, src, n, c0);
+        nn_rotate4(t, v, u, (d & 1) != 0, sg);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+          *(__nv_bfloat162*)(sa + wg_row(d * CIN + c0 + i) + wa[a]) =
+              __floats2bfloat162_rn(t[i * 3 + a].r, t[i * 3 + a].i);
+    }
+    // B: the delta rows of these sites, one output channel per warp
+    if (warp < COUT) {
+      const int o = warp;
+      cx<float> dl[3];
+      if (valid) {
+        const float4* ds = (const float4*)(delta + p * delta_half);
+        constexpr int NG = 3 * COUT / 2;
+        // complex index o*3 + a lives in group (o*3 + a) / 2, half (o*3 + a) % 2
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+          const int ci = o * 3 + a;
+          const float4 q = __ldg(ds + sbi(cb, ci >> 1, NG));
+          dl[a] = (ci & 1) ? mk<float>(q.z, q.w) : mk<float>(q.x, q.y);
         }
+      } else {
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
+        for (int a = 0; a < 3; a++) dl[a] = mk<float>(0.f, 0.f);
+      }
 #pragma unroll
-          for (int a = 0; a < 3; a++) {
-#pragma unroll
-            for (int part = 0; part < 2; part++) {
-              const int kp = (part * 3 + a) * WG_SITES + lane;
-              const float v = part ? t[i * 3 + a].i : t[i * 3 + a].r;
-              *(__nv_bfloat16*)(sa + (kp >> 4) * WG_ACH +
-                                kmajor_offset(d * CIN + c0 + i, kp & 15, 16)) =
-                  __float2bfloat16_rn(v);
-            }
-          }
-        }
+      for (int a = 0; a < 3; a++) {
+        *(__nv_bfloat162*)(sb + wg_row(2 * o) + wb[a]) = __floats2bfloat162_rn(dl[a].r, dl[a].i);
+        *(__nv_bfloat162*)(sb + wg_row(2 * o + 1) + wb[a]) =
+            __floats2bfloat162_rn(dl[a].i, -dl[a].r);
       }
     }
-    // B: the delta rows of these sites, output channels spread over the warps
-    // that do not transport (CIN = 4) or over all warps (CIN = 8)
-    {
-      constexpr int NW = SPLIT ? 8 : 4;
-      const int w0 = SPLIT ? warp : warp - 4;
-      if (w0 >= 0) {
-        for (int o = w0; o < COUT; o += NW) {
-          cx<float> dl[3];
-          if (valid) {
-            const float4* src = (const float4*)(delta + p * delta_half);
-            constexpr int NG = 3 * COUT / 2;
-            // complex index o*3 + a lives in group (o*3 + a) / 2, half (o*3 + a) % 2
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-              const int ci = o * 3 + a;
-              const float4 q = __ldg(src + sbi(cb, ci >> 1, NG));
-              dl[a] = (ci & 1) ? mk<float>(q.z, q.w) : mk<float>(q.x, q.y);
-            }
-          } else {
-#pragma unroll
-            for (int a = 0; a < 3; a++) dl[a] = mk<float>(0.f, 0.f);
-          }
-#pragma unroll
-          for (int a = 0; a < 3; a++) {
-            const cx<float> v = dl[a];
-            const int k0 = a * WG_SITES + lane, k1 = (3 + a) * WG_SITES + lane;
-            // Re G row: [delta_r | delta_i] ; Im G row: [delta_i | -delta_r]
-            *(__nv_bfloat16*)(sb + (k0 >> 4) * WG_BCH + kmajor_offset(2 * o, k0 & 15, 16)) =
-                __float2bfloat16_rn(v.r);
-            *(__nv_bfloat16*)(sb + (k1 >> 4) * WG_BCH + kmajor_offset(2 * o, k1 & 15, 16)) =
-                __float2bfloat16_rn(v.i);
-            *(__nv_bfloat16*)(sb + (k0 >> 4) * WG_BCH + kmajor_offset(2 * o + 1, k0 & 15, 16)) =
-                __float2bfloat16_rn(v.i);
-            *(__nv_bfloat16*)(sb + (k1 >> 4) * WG_BCH + kmajor_offset(2 * o + 1, k1 & 15, 16)) =
-                __float2bfloat16_rn(-v.r);
-          }
-        }
-      }
-    }
-      fence_smem_to_async();
+    fence_smem_to_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (tid == 0) {
       for (int kc = 0; kc < WG_KCH; kc++) {
-        const uint64_t ad = make_smem_desc(smem_u32(sa + kc * WG_ACH), 128, 256);
-        const uint64_t bd = make_smem_desc(smem_u32(sb + kc * WG_BCH), 128, 256);
+        const uint64_t ad = make_smem_desc(smem_u32(sa + kc * WG_ACH), WG_ALBO, WG_SBO);
+        const uint64_t bd = make_smem_desc(smem_u32(sb + kc * WG_BCH), WG_BLBO, WG_SBO);
         tc_mma_bf16(tbase, ad, bd, idesc, (G > 0 || kc > 0) ? 1u : 0u);
       }
       tc_commit(&bar[buf]);
@@ -323,7 +355,7 @@ __global__ void __launch_bounds__(WG_THREADS) nn_wgrad_tc_kernel(const NnLayerAr
 }
 
 // persistent grid of the tensor-core weight gradient: at most `cap` CTAs
-// (the caller's partial buffer), 2 per SM (two K buffers of 108 KB each CTA)
+// (the caller's partial buffer), 2 per SM (two K buffers, 112 KB a CTA)
 template <int CIN, int COUT>
 static cudaError_t launch_wgrad_tc(const NnLayerArgs& A, const char* delta, size_t dh,
                                    float* partials, int cap, int* grid_out, cudaStream_t st) {
@@ -370,7 +402,8 @@ static cudaError_t nn_wgrad(int cin, int cout, const Geom& g, const void* gauge,
     return cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
   const int n = NN_NDIR * cout * cin * 2;
-  nn_sum_tiles<<<(n + 127) / 128, 128, 0, st>>>(partials, grid, n, grad_out, accumulate);
+  nn_sum_tiles<<<(n + 31) / 32, dim3(32, NN_SUM_SLICES), 0, st>>>(partials, grid, n, grad_out,
+                                                                  accumulate);
   return cudaGetLastError();
 }
 

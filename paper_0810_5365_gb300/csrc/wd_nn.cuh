@@ -194,24 +194,9 @@ __device__ __forceinline__ void nn_nbr(int (&nb)[NN_NDIR], int& x3, int cb, int 
   nb[8] = x3 == 0 ? cb + (g.L[3] - 1) * g.S3 : cb - g.S3;
 }
 
-// T_d of four input channels at this site
-template <int C>
-__device__ __forceinline__ void nn_transport4(cx<float> (&t)[12], const NnLayerArgs& A, int d,
-                                              int p, int cb, int n, int x3, int c0) {
-  cx<float> v[12];
-  nn_load4<C>(v, A.in + (d == 0 ? p : 1 - p) * A.in_half, n, c0);
-  if (d == 0) {
-#pragma unroll
-    for (int k = 0; k < 12; k++) t[k] = v[k];
-    return;
-  }
-  const int mu = (d - 1) >> 1;
-  const bool fwd = (d & 1) != 0;
-  cx<float> u[9];
-  load_link<WD_F32, 12, float>(u, A.gauge, 2 * mu + (fwd ? p : 1 - p), fwd ? cb : n,
-                               A.g.Vh_pad);
-  const bool flip = mu == 3 && (fwd ? x3 == A.g.L[3] - 1 : x3 == 0);
-  const float sg = flip ? -1.f : 1.f;
+// t = sg U v (fwd) or sg U^+ v of four channels
+__device__ __forceinline__ void nn_rotate4(cx<float> (&t)[12], const cx<float> (&v)[12],
+                                           const cx<float> (&u)[9], bool fwd, float sg) {
 #pragma unroll
   for (int c = 0; c < 4; c++) {
 #pragma unroll
@@ -227,6 +212,34 @@ __device__ __forceinline__ void nn_transport4(cx<float> (&t)[12], const NnLayerA
       t[c * 3 + a] = sg * w;
     }
   }
+}
+
+// the link of direction d > 0 at this site (n its neighbour) and the
+// antiperiodic sign of the hop
+__device__ __forceinline__ float nn_link(cx<float> (&u)[9], const NnLayerArgs& A, int d, int p,
+                                         int cb, int n, int x3) {
+  const int mu = (d - 1) >> 1;
+  const bool fwd = (d & 1) != 0;
+  load_link<WD_F32, 12, float>(u, A.gauge, 2 * mu + (fwd ? p : 1 - p), fwd ? cb : n,
+                               A.g.Vh_pad);
+  const bool flip = mu == 3 && (fwd ? x3 == A.g.L[3] - 1 : x3 == 0);
+  return flip ? -1.f : 1.f;
+}
+
+// T_d of four input channels at this site
+template <int C>
+__device__ __forceinline__ void nn_transport4(cx<float> (&t)[12], const NnLayerArgs& A, int d,
+                                              int p, int cb, int n, int x3, int c0) {
+  cx<float> v[12];
+  nn_load4<C>(v, A.in + (d == 0 ? p : 1 - p) * A.in_half, n, c0);
+  if (d == 0) {
+#pragma unroll
+    for (int k = 0; k < 12; k++) t[k] = v[k];
+    return;
+  }
+  cx<float> u[9];
+  const float sg = nn_link(u, A, d, p, cb, n, x3);
+  nn_rotate4(t, v, u, (d & 1) != 0, sg);
 }
 
 // ---------------------------------------------------------------------------
