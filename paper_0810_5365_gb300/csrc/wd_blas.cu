@@ -33,7 +33,7 @@ int num_sms() {
 
 int blas_grid(long long n, int bs) {
   long long need = (n + bs - 1) / bs;
-  long long cap = (long long)num_sms() * 8;
+  long long cap = (long long)num_sms() * (2048 / bs);
   if (need < 1) need = 1;
   return (int)(need < cap ? need : cap);
 }
@@ -140,47 +140,119 @@ RedScratch scratch() {
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ int lex_parity(int i, const Geom& g) {
-  int x0 = i % g.L[0];
-  int r = i / g.L[0];
-  int x1 = r % g.L[1];
-  r /= g.L[1];
-  int x2 = r % g.L[2];
-  int x3 = r / g.L[2];
-  return (x0 + x1 + x2 + x3) & 1;
+  const int r0 = fdiv(i >> 1, g.dLh0);  // i / L0 (L0 is even)
+  const int r1 = fdiv(r0, g.dL1);
+  const int x3 = fdiv(r1, g.dL2);
+  return (i + (r0 - r1 * g.L[1]) + (r1 - x3 * g.L[2]) + x3) & 1;
+}
+
+// The canonical side of the conversions holds 192 (spinor) or 144 (link)
+// consecutive bytes per site, which one thread per site would touch 16 bytes
+// at a time, 192 or 144 bytes apart from its neighbour: a warp's request then
+// covers 32 sectors half full.  Here a warp moves its 32 sites between
+// canonical memory and shared memory in whole lines, and each thread takes
+// its site from there (an odd number of 16-byte words per site, so that the
+// eight lanes of a phase use different banks).  The packing kernels copy the
+// next 32 sites (cp.async, no registers) while they convert the current ones.
+//
+// 24^3x48, us, one thread per site on canonical memory (and conversions on the
+// FP64 pipe, wd_common.cuh) -> now:
+//   links   F32 12-real 90 -> 80, 18-real 101 -> 88; F16 90 -> 72;
+//           F64 12-real 114 -> 98, 18-real 144 -> 116   (HBM: 75 for F32 12-real)
+//   pack    F32 42 -> 35, F16 34 -> 32, F64 46 -> 41     (28 for F32)
+//   unpack  F32 88 -> 33, F16 94 -> 29, F64 106 -> 49    (28 for F32)
+// Without the asynchronous copies the links of F32 18-real took 127.
+constexpr int CANON_BS = 96;  // three warps: two buffers each within 48 KB
+
+__device__ __forceinline__ void cp_async16(double2* dst, const double2* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// all but the newest N groups of this thread have arrived
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory");
+}
+
+// NC of every SW canonical words of the sites i0 .. i0 + 31 (below n), NS
+// words apart in w
+template <int NC, int SW, int NS>
+__device__ __forceinline__ void stage_sites(double2* w, const double2* src, long long i0,
+                                            long long n, int lane) {
+  if (i0 < n) {
+    const int words = NC * (int)(n - i0 < 32 ? n - i0 : 32);
+#pragma unroll
+    for (int j = 0; j < NC; j++) {
+      const int e = lane + 32 * j;
+      if (e < words) cp_async16(w + e / NC * NS + e % NC, src + (i0 + e / NC) * SW + e % NC);
+    }
+  }
+  cp_async_commit();
 }
 
 // src: canonical complex double [n][12]; half layout (full = 0) indexes by cb,
 // full layout (full = 1) by lexicographic site.
 template <int P>
-__global__ void pack_spinor_kernel(char* dst, const double2* __restrict__ src, Geom g, int full,
-                                   size_t half_bytes) {
-  long long n = full ? 2LL * g.Vh : g.Vh;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    int cb = full ? (int)(i >> 1) : (int)i;
-    int par = full ? lex_parity((int)i, g) : 0;
-    cx<double> s[12];
+__global__ void __launch_bounds__(CANON_BS)
+    pack_spinor_kernel(char* dst, const double2* __restrict__ src, Geom g, int full,
+                       size_t half_bytes) {
+  __shared__ double2 sm[CANON_BS / 32][2][32 * 13];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long n = full ? 2LL * g.Vh : g.Vh;
+  const long long step = (long long)gridDim.x * CANON_BS;
+  long long i0 = blockIdx.x * (long long)CANON_BS + 32 * warp;
+  stage_sites<12, 12, 13>(sm[warp][0], src, i0, n, lane);
+  for (int b = 0; i0 < n; i0 += step, b ^= 1) {
+    stage_sites<12, 12, 13>(sm[warp][b ^ 1], src, i0 + step, n, lane);
+    cp_async_wait<1>();
+    __syncwarp();
+    const double2* w = sm[warp][b];
+    const long long i = i0 + lane;
+    if (i < n) {
+      const int cb = full ? (int)(i >> 1) : (int)i;
+      const int par = full ? lex_parity((int)i, g) : 0;
+      cx<double> s[12];
 #pragma unroll
-    for (int k = 0; k < 12; k++) {
-      double2 v = src[i * 12 + k];
-      s[k] = mk<double>(v.x, v.y);
+      for (int k = 0; k < 12; k++) {
+        const double2 q = w[lane * 13 + k];
+        s[k] = mk<double>(q.x, q.y);
+      }
+      store_spinor<P, double>(dst + par * half_bytes, cb, g.Vh_pad, s);
     }
-    store_spinor<P, double>(dst + par * half_bytes, cb, g.Vh_pad, s);
+    __syncwarp();  // (the next copy into this buffer follows)
   }
 }
 
 template <int P>
-__global__ void unpack_spinor_kernel(double2* dst, const char* __restrict__ src, Geom g, int full,
-                                     size_t half_bytes) {
-  long long n = full ? 2LL * g.Vh : g.Vh;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    int cb = full ? (int)(i >> 1) : (int)i;
-    int par = full ? lex_parity((int)i, g) : 0;
-    cx<double> s[12];
-    load_spinor_rw<P, double>(s, src + par * half_bytes, cb, g.Vh_pad);
+__global__ void __launch_bounds__(CANON_BS)
+    unpack_spinor_kernel(double2* dst, const char* __restrict__ src, Geom g, int full,
+                         size_t half_bytes) {
+  __shared__ double2 sm[CANON_BS / 32][32 * 13];
+  const int lane = threadIdx.x & 31;
+  double2* w = sm[threadIdx.x >> 5];
+  const long long n = full ? 2LL * g.Vh : g.Vh;
+  const long long step = (long long)gridDim.x * CANON_BS;
+  for (long long i0 = blockIdx.x * (long long)CANON_BS + (threadIdx.x & ~31); i0 < n; i0 += step) {
+    const int words = 12 * (int)(n - i0 < 32 ? n - i0 : 32);
+    const long long i = i0 + lane;
+    if (i < n) {
+      const int cb = full ? (int)(i >> 1) : (int)i;
+      const int par = full ? lex_parity((int)i, g) : 0;
+      cx<double> s[12];
+      load_spinor_rw<P, double>(s, src + par * half_bytes, cb, g.Vh_pad);
 #pragma unroll
-    for (int k = 0; k < 12; k++) dst[i * 12 + k] = make_double2(s[k].r, s[k].i);
+      for (int k = 0; k < 12; k++) w[lane * 13 + k] = make_double2(s[k].r, s[k].i);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 12; j++) {
+      const int e = lane + 32 * j;
+      if (e < words) dst[i0 * 12 + e] = w[e + e / 12];
+    }
+    __syncwarp();
   }
 }
 
@@ -196,9 +268,9 @@ cudaError_t pack_spinor(void* dst, const double* src, const Geom& g, int parity,
                         cudaStream_t st) {
   int full = parity == WD_FULL;
   long long n = full ? 2LL * g.Vh : g.Vh;
-  int grid = blas_grid(n, 256);
+  int grid = blas_grid(n, CANON_BS);
   size_t hb = spinor_half_bytes(g, prec);
-  WD_PREC_SWITCH(prec, pack_spinor_kernel, grid, 256, 0, st>>>((char*)dst, (const double2*)src, g,
+  WD_PREC_SWITCH(prec, pack_spinor_kernel, grid, CANON_BS, 0, st>>>((char*)dst, (const double2*)src, g,
                                                                 full, hb))
   return cudaGetLastError();
 }
@@ -207,9 +279,9 @@ cudaError_t unpack_spinor(double* dst, const void* src, const Geom& g, int parit
                           cudaStream_t st) {
   int full = parity == WD_FULL;
   long long n = full ? 2LL * g.Vh : g.Vh;
-  int grid = blas_grid(n, 256);
+  int grid = blas_grid(n, CANON_BS);
   size_t hb = spinor_half_bytes(g, prec);
-  WD_PREC_SWITCH(prec, unpack_spinor_kernel, grid, 256, 0, st>>>((double2*)dst, (const char*)src,
+  WD_PREC_SWITCH(prec, unpack_spinor_kernel, grid, CANON_BS, 0, st>>>((double2*)dst, (const char*)src,
                                                                   g, full, hb))
   return cudaGetLastError();
 }
@@ -218,27 +290,31 @@ cudaError_t unpack_spinor(double* dst, const void* src, const Geom& g, int parit
 // gauge packing
 // ---------------------------------------------------------------------------
 
+// the RC / 2 stored entries of a link
 template <int P, int RC>
 __device__ __forceinline__ void store_link(char* gauge, int region, int cb, int Vh_pad,
-                                           const cx<double> (&u)[9]) {
+                                           const cx<double> (&u)[RC / 2]) {
   if constexpr (P == WD_F64) {
-    constexpr int NC = RC == 18 ? 9 : 6;
+    constexpr int NC = RC / 2;
     double2* p = (double2*)gauge + (size_t)region * Vh_pad * NC;
 #pragma unroll
     for (int k = 0; k < NC; k++) p[sbi(cb, k, NC)] = make_double2(u[k].r, u[k].i);
-  } else if constexpr (P == WD_F32) {
+    return;
+  }
+  cx<float> w[RC / 2];
+  convert(w, u);
+  if constexpr (P == WD_F32) {
     if constexpr (RC == 18) {
       float2* p = (float2*)gauge + (size_t)region * Vh_pad * 9;
 #pragma unroll
-      for (int k = 0; k < 9; k++) p[sbi(cb, k, 9)] = make_float2((float)u[k].r, (float)u[k].i);
+      for (int k = 0; k < 9; k++) p[sbi(cb, k, 9)] = make_float2(w[k].r, w[k].i);
     } else {
       float4* p = (float4*)gauge + (size_t)region * Vh_pad * 3;
 #pragma unroll
       for (int k = 0; k < 3; k++)
-        p[sbi(cb, k, 3)] = make_float4((float)u[2 * k].r, (float)u[2 * k].i,
-                                       (float)u[2 * k + 1].r, (float)u[2 * k + 1].i);
+        p[sbi(cb, k, 3)] = make_float4(w[2 * k].r, w[2 * k].i, w[2 * k + 1].r, w[2 * k + 1].i);
     }
-  } else {
+  } else if constexpr (P == WD_F16) {
     int4* pa = (int4*)gauge + (size_t)region * Vh_pad;
     int2* pb = (int2*)(gauge + (size_t)8 * Vh_pad * 16) + (size_t)region * Vh_pad;
     int4 a;
@@ -246,44 +322,59 @@ __device__ __forceinline__ void store_link(char* gauge, int region, int cb, int 
     __half2* ha = reinterpret_cast<__half2*>(&a);
     __half2* hb = reinterpret_cast<__half2*>(&b);
 #pragma unroll
-    for (int j = 0; j < 4; j++) ha[j] = __floats2half2_rn((float)u[j].r, (float)u[j].i);
+    for (int j = 0; j < 4; j++) ha[j] = __floats2half2_rn(w[j].r, w[j].i);
 #pragma unroll
-    for (int j = 0; j < 2; j++) hb[j] = __floats2half2_rn((float)u[4 + j].r, (float)u[4 + j].i);
+    for (int j = 0; j < 2; j++) hb[j] = __floats2half2_rn(w[4 + j].r, w[4 + j].i);
     pa[sbi(cb, 0, 1)] = a;
     pb[sbi(cb, 0, 1)] = b;
   }
 }
 
-// src: canonical [4][V][3][3] complex double; one thread per (mu, site)
+// src: canonical [4][V][3][3] complex double; one thread per (mu, site), the
+// warp's links staged as the spinors above (of 12-real storage the first two
+// rows only)
 template <int P, int RC>
-__global__ void pack_gauge_kernel(char* dst, const double2* __restrict__ src, Geom g) {
-  long long V = 2LL * g.Vh;
-  long long n = 4 * V;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    int mu = (int)(t / V);
-    int i = (int)(t - mu * V);
-    int par = lex_parity(i, g);
-    cx<double> u[9];
+__global__ void __launch_bounds__(CANON_BS)
+    pack_gauge_kernel(char* dst, const double2* __restrict__ src, Geom g) {
+  constexpr int NC = RC / 2, NS = NC | 1;  // words read per link, words between links
+  __shared__ double2 sm[CANON_BS / 32][2][32 * NS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long V = 2LL * g.Vh, n = 4 * V;
+  const long long step = (long long)gridDim.x * CANON_BS;
+  long long t0 = blockIdx.x * (long long)CANON_BS + 32 * warp;
+  stage_sites<NC, 9, NS>(sm[warp][0], src, t0, n, lane);
+  for (int b = 0; t0 < n; t0 += step, b ^= 1) {
+    stage_sites<NC, 9, NS>(sm[warp][b ^ 1], src, t0 + step, n, lane);
+    cp_async_wait<1>();
+    __syncwarp();
+    const double2* w = sm[warp][b];
+    const long long t = t0 + lane;
+    if (t < n) {
+      const int mu = (int)(t / V);
+      const int i = (int)(t - mu * V);
+      const int par = lex_parity(i, g);
+      cx<double> u[NC];
 #pragma unroll
-    for (int k = 0; k < 9; k++) {
-      double2 v = src[t * 9 + k];
-      u[k] = mk<double>(v.x, v.y);
+      for (int k = 0; k < NC; k++) {
+        const double2 q = w[lane * NS + k];
+        u[k] = mk<double>(q.x, q.y);
+      }
+      store_link<P, RC>(dst, 2 * mu + par, i >> 1, g.Vh_pad, u);
     }
-    store_link<P, RC>(dst, 2 * mu + par, i >> 1, g.Vh_pad, u);
+    __syncwarp();  // (the next copy into this buffer follows)
   }
 }
 
 cudaError_t pack_gauge(void* dst, const double* src, const Geom& g, int prec, int recon,
                        cudaStream_t st) {
-  int grid = blas_grid(8LL * g.Vh, 256);
+  int grid = blas_grid(8LL * g.Vh, CANON_BS);
   const double2* s = (const double2*)src;
   char* d = (char*)dst;
-  if (prec == WD_F64 && recon == 18) pack_gauge_kernel<WD_F64, 18><<<grid, 256, 0, st>>>(d, s, g);
-  else if (prec == WD_F64 && recon == 12) pack_gauge_kernel<WD_F64, 12><<<grid, 256, 0, st>>>(d, s, g);
-  else if (prec == WD_F32 && recon == 18) pack_gauge_kernel<WD_F32, 18><<<grid, 256, 0, st>>>(d, s, g);
-  else if (prec == WD_F32 && recon == 12) pack_gauge_kernel<WD_F32, 12><<<grid, 256, 0, st>>>(d, s, g);
-  else if (prec == WD_F16 && recon == 12) pack_gauge_kernel<WD_F16, 12><<<grid, 256, 0, st>>>(d, s, g);
+  if (prec == WD_F64 && recon == 18) pack_gauge_kernel<WD_F64, 18><<<grid, CANON_BS, 0, st>>>(d, s, g);
+  else if (prec == WD_F64 && recon == 12) pack_gauge_kernel<WD_F64, 12><<<grid, CANON_BS, 0, st>>>(d, s, g);
+  else if (prec == WD_F32 && recon == 18) pack_gauge_kernel<WD_F32, 18><<<grid, CANON_BS, 0, st>>>(d, s, g);
+  else if (prec == WD_F32 && recon == 12) pack_gauge_kernel<WD_F32, 12><<<grid, CANON_BS, 0, st>>>(d, s, g);
+  else if (prec == WD_F16 && recon == 12) pack_gauge_kernel<WD_F16, 12><<<grid, CANON_BS, 0, st>>>(d, s, g);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

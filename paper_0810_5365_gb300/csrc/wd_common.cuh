@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -228,6 +229,77 @@ __device__ __forceinline__ T ldin(const T* p) {
     return __ldg(p);
 }
 
+// float <-> double on the integer pipe, with the results of the conversion
+// instructions (round to nearest even).  Those run on GB300's FP64 pipe, at
+// 1/64 of the FP32 rate: the 24 of a site took longer than its memory traffic
+// (packing links to FP32: 64 % of that pipe busy, also where they were
+// predicated off).  Normal numbers and zeros are done here; a site that holds
+// anything else takes the instructions, in a branch of its own.
+__host__ __device__ __forceinline__ bool narrows(double d) {  // zero, or in [2^-126, 2^128)
+  unsigned long long r;
+  memcpy(&r, &d, 8);
+  const unsigned a = (unsigned)(r >> 32) & 0x7fffffffu;
+  return a - 0x38100000u < 0x0fe00000u || (a | (unsigned)r) == 0u;
+}
+__host__ __device__ __forceinline__ float narrow(double d) {
+  unsigned long long r;
+  memcpy(&r, &d, 8);
+  const unsigned hi = (unsigned)(r >> 32), lo = (unsigned)r, a = hi & 0x7fffffffu;
+  const unsigned m = ((a - 0x38000000u) << 3) | (lo >> 29), rem = lo << 3;
+  const unsigned up = (rem > 0x80000000u || (rem == 0x80000000u && (m & 1u))) ? 1u : 0u;
+  const unsigned b = (hi & 0x80000000u) | ((a | lo) == 0u ? 0u : m + up);
+  float f;
+  memcpy(&f, &b, 4);
+  return f;
+}
+__host__ __device__ __forceinline__ bool widens(float f) {  // zero or normal
+  unsigned b;
+  memcpy(&b, &f, 4);
+  b &= 0x7fffffffu;
+  return b - 0x00800000u < 0x7f000000u || b == 0u;
+}
+__host__ __device__ __forceinline__ double widen(float f) {
+  unsigned b;
+  memcpy(&b, &f, 4);
+  const unsigned a = b & 0x7fffffffu;
+  const unsigned hi = a == 0u ? b : (b & 0x80000000u) | ((a >> 3) + 0x38000000u), lo = b << 29;
+  const unsigned long long r = ((unsigned long long)hi << 32) | lo;
+  double d;
+  memcpy(&d, &r, 8);
+  return d;
+}
+template <int N>
+__host__ __device__ __forceinline__ void convert(cx<float> (&o)[N], const cx<double> (&s)[N]) {
+  bool plain = true;
+#pragma unroll
+  for (int k = 0; k < N; k++) plain = plain && narrows(s[k].r) && narrows(s[k].i);
+  if (plain) {
+#pragma unroll
+    for (int k = 0; k < N; k++) o[k].r = narrow(s[k].r), o[k].i = narrow(s[k].i);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; k++) o[k].r = (float)s[k].r, o[k].i = (float)s[k].i;
+  }
+}
+template <int N>
+__host__ __device__ __forceinline__ void convert(cx<double> (&o)[N], const cx<float> (&s)[N]) {
+  bool plain = true;
+#pragma unroll
+  for (int k = 0; k < N; k++) plain = plain && widens(s[k].r) && widens(s[k].i);
+  if (plain) {
+#pragma unroll
+    for (int k = 0; k < N; k++) o[k].r = widen(s[k].r), o[k].i = widen(s[k].i);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; k++) o[k].r = (double)s[k].r, o[k].i = (double)s[k].i;
+  }
+}
+template <typename R, int N>
+__host__ __device__ __forceinline__ void convert(cx<R> (&o)[N], const cx<R> (&s)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; k++) o[k] = s[k];
+}
+
 // Load the 12 complex components of site cb as type R.
 template <int P, typename R, bool COH = false>
 __device__ __forceinline__ void load_spinor(cx<R> (&s)[12], const void* base, int cb, int Vh_pad) {
@@ -269,23 +341,28 @@ template <int P, typename R>
 __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base, int cb, int Vh_pad) {
   if constexpr (P == WD_F64) {
     const double2* p = (const double2*)base;
+    cx<double> w[12];
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       double2 v = p[sbi(cb, k, 12)];
-      s[k] = mk<R>((R)v.x, (R)v.y);
+      w[k] = mk<double>(v.x, v.y);
     }
+    convert(s, w);
   } else if constexpr (P == WD_F32) {
     const float4* p = (const float4*)base;
+    cx<float> w[12];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
       float4 v = p[sbi(cb, k, 6)];
-      s[2 * k] = mk<R>((R)v.x, (R)v.y);
-      s[2 * k + 1] = mk<R>((R)v.z, (R)v.w);
+      w[2 * k] = mk<float>(v.x, v.y);
+      w[2 * k + 1] = mk<float>(v.z, v.w);
     }
+    convert(s, w);
   } else {
     const int4* p = (const int4*)base;
     const float* sc = (const float*)((const char*)base + (size_t)Vh_pad * 48);
     float scale = sc[cb];
+    cx<float> w[12];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       int4 v = p[sbi(cb, k, 3)];
@@ -293,9 +370,10 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
 #pragma unroll
       for (int j = 0; j < 4; j++) {
         float2 f = __half22float2(h[j]);
-        s[4 * k + j] = mk<R>((R)(f.x * scale), (R)(f.y * scale));
+        w[4 * k + j] = mk<float>(f.x * scale, f.y * scale);
       }
     }
+    convert(s, w);
   }
 }
 
@@ -306,8 +384,10 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
 template <typename R, bool KEEP>
 __device__ __forceinline__ void store_spinor_f16(void* base, int cb, int Vh_pad, cx<R> (&s)[12]) {
   float m = 0.f;
+  cx<float> w[12];
+  convert(w, s);
 #pragma unroll
-  for (int k = 0; k < 12; k++) m = fmaxf(m, fmaxf(fabsf((float)s[k].r), fabsf((float)s[k].i)));
+  for (int k = 0; k < 12; k++) m = fmaxf(m, fmaxf(fabsf(w[k].r), fabsf(w[k].i)));
   float inv = m > 0.f ? 1.0f / m : 0.f;
   int4* p = (int4*)base;
   float* sc = (float*)((char*)base + (size_t)Vh_pad * 48);
@@ -317,7 +397,7 @@ __device__ __forceinline__ void store_spinor_f16(void* base, int cb, int Vh_pad,
     __half2* h = reinterpret_cast<__half2*>(&v);
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      h[j] = __floats2half2_rn((float)s[4 * k + j].r * inv, (float)s[4 * k + j].i * inv);
+      h[j] = __floats2half2_rn(w[4 * k + j].r * inv, w[4 * k + j].i * inv);
       if constexpr (KEEP) {
         const float2 f = __half22float2(h[j]);
         s[4 * k + j] = mk<R>((R)(f.x * m), (R)(f.y * m));
@@ -332,14 +412,17 @@ template <int P, typename R>
 __device__ __forceinline__ void store_spinor(void* base, int cb, int Vh_pad, const cx<R> (&s)[12]) {
   if constexpr (P == WD_F64) {
     double2* p = (double2*)base;
+    cx<double> w[12];
+    convert(w, s);
 #pragma unroll
-    for (int k = 0; k < 12; k++) p[sbi(cb, k, 12)] = make_double2((double)s[k].r, (double)s[k].i);
+    for (int k = 0; k < 12; k++) p[sbi(cb, k, 12)] = make_double2(w[k].r, w[k].i);
   } else if constexpr (P == WD_F32) {
     float4* p = (float4*)base;
+    cx<float> w[12];
+    convert(w, s);
 #pragma unroll
     for (int k = 0; k < 6; k++)
-      p[sbi(cb, k, 6)] = make_float4((float)s[2 * k].r, (float)s[2 * k].i,
-                                     (float)s[2 * k + 1].r, (float)s[2 * k + 1].i);
+      p[sbi(cb, k, 6)] = make_float4(w[2 * k].r, w[2 * k].i, w[2 * k + 1].r, w[2 * k + 1].i);
   } else {
     store_spinor_f16<R, false>(base, cb, Vh_pad, const_cast<cx<R>(&)[12]>(s));
   }
