@@ -294,11 +294,18 @@ __host__ __device__ __forceinline__ void convert(cx<double> (&o)[N], const cx<fl
     for (int k = 0; k < N; k++) o[k].r = (double)s[k].r, o[k].i = (double)s[k].i;
   }
 }
-template <typename R, int N>
-__host__ __device__ __forceinline__ void convert(cx<R> (&o)[N], const cx<R> (&s)[N]) {
-#pragma unroll
-  for (int k = 0; k < N; k++) o[k] = s[k];
+// The array that values of type T go through on their way to or from s: s
+// itself when it has that type (then the conversion is nothing), else tmp.
+template <typename T, int N>
+__host__ __device__ __forceinline__ cx<T> (&through(cx<T> (&s)[N], cx<T> (&)[N]))[N] {
+  return s;
 }
+template <typename T, typename R, int N>
+__host__ __device__ __forceinline__ cx<T> (&through(cx<R> (&)[N], cx<T> (&tmp)[N]))[N] {
+  return tmp;
+}
+template <typename R, int N>
+__host__ __device__ __forceinline__ void convert(cx<R> (&)[N], const cx<R> (&)[N]) {}
 
 // Load the 12 complex components of site cb as type R.
 template <int P, typename R, bool COH = false>
@@ -341,7 +348,8 @@ template <int P, typename R>
 __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base, int cb, int Vh_pad) {
   if constexpr (P == WD_F64) {
     const double2* p = (const double2*)base;
-    cx<double> w[12];
+    cx<double> tmp[12];
+    auto& w = through<double>(s, tmp);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       double2 v = p[sbi(cb, k, 12)];
@@ -350,7 +358,8 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
     convert(s, w);
   } else if constexpr (P == WD_F32) {
     const float4* p = (const float4*)base;
-    cx<float> w[12];
+    cx<float> tmp[12];
+    auto& w = through<float>(s, tmp);
 #pragma unroll
     for (int k = 0; k < 6; k++) {
       float4 v = p[sbi(cb, k, 6)];
@@ -362,7 +371,8 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
     const int4* p = (const int4*)base;
     const float* sc = (const float*)((const char*)base + (size_t)Vh_pad * 48);
     float scale = sc[cb];
-    cx<float> w[12];
+    cx<float> tmp[12];
+    auto& w = through<float>(s, tmp);
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       int4 v = p[sbi(cb, k, 3)];
@@ -377,6 +387,77 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
   }
 }
 
+// One site of a packed field as it sits in memory (the format load_spinor_rw
+// reads), so that a kernel can issue the loads of its next site before it
+// computes the current one.
+template <int P>
+struct RawSite;
+template <>
+struct RawSite<WD_F16> {
+  int4 v[3];
+  float s;
+};
+template <>
+struct RawSite<WD_F32> {
+  float4 v[6];
+};
+template <>
+struct RawSite<WD_F64> {
+  double2 v[12];
+};
+
+template <int P>
+__device__ __forceinline__ void load_raw(RawSite<P>& o, const void* base, int cb, int Vh_pad) {
+  if constexpr (P == WD_F16) {
+    const int4* p = (const int4*)base;
+#pragma unroll
+    for (int k = 0; k < 3; k++) o.v[k] = p[sbi(cb, k, 3)];
+    o.s = ((const float*)((const char*)base + (size_t)Vh_pad * 48))[cb];
+  } else if constexpr (P == WD_F32) {
+    const float4* p = (const float4*)base;
+#pragma unroll
+    for (int k = 0; k < 6; k++) o.v[k] = p[sbi(cb, k, 6)];
+  } else {
+    const double2* p = (const double2*)base;
+#pragma unroll
+    for (int k = 0; k < 12; k++) o.v[k] = p[sbi(cb, k, 12)];
+  }
+}
+
+// the values of a raw site, with the arithmetic of load_spinor_rw
+template <int P, typename R>
+__device__ __forceinline__ void unpack_raw(cx<R> (&s)[12], const RawSite<P>& o) {
+  if constexpr (P == WD_F16) {
+    cx<float> tmp[12];
+    auto& w = through<float>(s, tmp);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const __half2* h = reinterpret_cast<const __half2*>(&o.v[k]);
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const float2 f = __half22float2(h[j]);
+        w[4 * k + j] = mk<float>(f.x * o.s, f.y * o.s);
+      }
+    }
+    convert(s, w);
+  } else if constexpr (P == WD_F32) {
+    cx<float> tmp[12];
+    auto& w = through<float>(s, tmp);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      w[2 * k] = mk<float>(o.v[k].x, o.v[k].y);
+      w[2 * k + 1] = mk<float>(o.v[k].z, o.v[k].w);
+    }
+    convert(s, w);
+  } else {
+    cx<double> tmp[12];
+    auto& w = through<double>(s, tmp);
+#pragma unroll
+    for (int k = 0; k < 12; k++) w[k] = mk<double>(o.v[k].x, o.v[k].y);
+    convert(s, w);
+  }
+}
+
 // An FP16 site: the values scaled by the site's largest |real component| m,
 // rounded to half, and m as the site scale.  KEEP: s is overwritten with
 // what was stored (the rounded values times m, as load_spinor_rw would read
@@ -384,7 +465,8 @@ __device__ __forceinline__ void load_spinor_rw(cx<R> (&s)[12], const void* base,
 template <typename R, bool KEEP>
 __device__ __forceinline__ void store_spinor_f16(void* base, int cb, int Vh_pad, cx<R> (&s)[12]) {
   float m = 0.f;
-  cx<float> w[12];
+  cx<float> tmp[12];
+  auto& w = through<float>(s, tmp);
   convert(w, s);
 #pragma unroll
   for (int k = 0; k < 12; k++) m = fmaxf(m, fmaxf(fabsf(w[k].r), fabsf(w[k].i)));
@@ -409,22 +491,26 @@ __device__ __forceinline__ void store_spinor_f16(void* base, int cb, int Vh_pad,
 }
 
 template <int P, typename R>
-__device__ __forceinline__ void store_spinor(void* base, int cb, int Vh_pad, const cx<R> (&s)[12]) {
+__device__ __forceinline__ void store_spinor(void* base, int cb, int Vh_pad,
+                                             const cx<R> (&site)[12]) {
+  cx<R>(&s)[12] = const_cast<cx<R>(&)[12]>(site);  // (not written)
   if constexpr (P == WD_F64) {
     double2* p = (double2*)base;
-    cx<double> w[12];
+    cx<double> tmp[12];
+    auto& w = through<double>(s, tmp);
     convert(w, s);
 #pragma unroll
     for (int k = 0; k < 12; k++) p[sbi(cb, k, 12)] = make_double2(w[k].r, w[k].i);
   } else if constexpr (P == WD_F32) {
     float4* p = (float4*)base;
-    cx<float> w[12];
+    cx<float> tmp[12];
+    auto& w = through<float>(s, tmp);
     convert(w, s);
 #pragma unroll
     for (int k = 0; k < 6; k++)
       p[sbi(cb, k, 6)] = make_float4(w[2 * k].r, w[2 * k].i, w[2 * k + 1].r, w[2 * k + 1].i);
   } else {
-    store_spinor_f16<R, false>(base, cb, Vh_pad, const_cast<cx<R>(&)[12]>(s));
+    store_spinor_f16<R, false>(base, cb, Vh_pad, s);
   }
 }
 

@@ -163,6 +163,24 @@ int num_sms();
 // grid of the grid-stride BLAS/reduction kernels for n sites
 int blas_grid(long long n, int bs);
 
+// CTAs of 256 threads of a kernel that are resident on an SM at once
+template <typename K>
+int ctas_per_sm(K kernel) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, 256, 0) != cudaSuccess || n < 1)
+    n = 1;
+  return n;
+}
+// The grid of a streaming kernel with 256-thread CTAs, one site per thread
+// and step: at most the resident CTAs, and no more of them than spread the
+// steps evenly, so that the last step is not a few stragglers' alone.
+inline int resident_grid(int per_sm, long long sites) {
+  const long long cap = (long long)per_sm * num_sms();
+  const long long need = sites > 0 ? (sites + 255) / 256 : 1;
+  const long long steps = (need + cap - 1) / cap;
+  return (int)((need + steps - 1) / steps);
+}
+
 // ---------------------------------------------------------------------------
 // layout and BLAS (wd_blas.cu)
 // ---------------------------------------------------------------------------

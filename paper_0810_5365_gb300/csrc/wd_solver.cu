@@ -51,68 +51,6 @@ __host__ __device__ __forceinline__ void zdiv(double ar, double ai, double br, d
   ci = (ai * br - ar * bi) / d;
 }
 
-// One site of a packed field as it sits in memory (the format load_spinor_rw
-// reads), so that a kernel can issue the loads of its next site before it
-// computes the current one.
-template <int P>
-struct RawSite;
-template <>
-struct RawSite<WD_F16> {
-  int4 v[3];
-  float s;
-};
-template <>
-struct RawSite<WD_F32> {
-  float4 v[6];
-};
-template <>
-struct RawSite<WD_F64> {
-  double2 v[12];
-};
-
-template <int P>
-__device__ __forceinline__ void load_raw(RawSite<P>& o, const void* base, int cb, int Vh_pad) {
-  if constexpr (P == WD_F16) {
-    const int4* p = (const int4*)base;
-#pragma unroll
-    for (int k = 0; k < 3; k++) o.v[k] = p[sbi(cb, k, 3)];
-    o.s = ((const float*)((const char*)base + (size_t)Vh_pad * 48))[cb];
-  } else if constexpr (P == WD_F32) {
-    const float4* p = (const float4*)base;
-#pragma unroll
-    for (int k = 0; k < 6; k++) o.v[k] = p[sbi(cb, k, 6)];
-  } else {
-    const double2* p = (const double2*)base;
-#pragma unroll
-    for (int k = 0; k < 12; k++) o.v[k] = p[sbi(cb, k, 12)];
-  }
-}
-
-// the values of a raw site, with the arithmetic of load_spinor_rw
-template <int P, typename R>
-__device__ __forceinline__ void unpack_raw(cx<R> (&s)[12], const RawSite<P>& o) {
-  if constexpr (P == WD_F16) {
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const __half2* h = reinterpret_cast<const __half2*>(&o.v[k]);
-#pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const float2 f = __half22float2(h[j]);
-        s[4 * k + j] = mk<R>((R)(f.x * o.s), (R)(f.y * o.s));
-      }
-    }
-  } else if constexpr (P == WD_F32) {
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      s[2 * k] = mk<R>((R)o.v[k].x, (R)o.v[k].y);
-      s[2 * k + 1] = mk<R>((R)o.v[k].z, (R)o.v[k].w);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; k++) s[k] = mk<R>((R)o.v[k].x, (R)o.v[k].y);
-  }
-}
-
 // The CG vector updates (and BiCGstab's p and s updates below) stream a few
 // fields once, about 10-20 us per call on 24^3x48.  They run on a grid of resident CTAs only (update_grid)
 // and each thread loads its next site before it computes the current one,
@@ -205,20 +143,6 @@ __global__ void __launch_bounds__(BS, (P == WD_F16 ? 2 : 1))
     rx = nxr;
   }
 }
-
-// The grid of an update kernel: as many CTAs of 256 threads as are resident
-// at once (the occupancy query), at most one per 256 sites.
-template <typename K>
-static int resident_grid(K kernel, int vh) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, 0) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  const long long need = (vh + 255) / 256;
-  const long long cap = (long long)per_sm * num_sms();
-  return (int)(need < cap ? need : cap);
-}
-
 
 // x64 += xs ; xs = 0
 template <int PX, int BS>
@@ -456,11 +380,11 @@ __global__ void bicg_restart_scalars(CgScalars* sc) {
 
 template <int P, int PX>
 static void update_grids_t(int vh, int (&grid)[5]) {
-  grid[0] = resident_grid(cg_update_r<P, 256>, vh);
-  grid[1] = resident_grid(cg_update_xp<P, PX, 256>, vh);
-  grid[2] = resident_grid(bicg_update_p<P, 256>, vh);
-  grid[3] = resident_grid(bicg_update_s<P, 256>, vh);
-  grid[4] = resident_grid(bicg_update_xr<P, PX, 256>, vh);
+  grid[0] = resident_grid(ctas_per_sm(cg_update_r<P, 256>), vh);
+  grid[1] = resident_grid(ctas_per_sm(cg_update_xp<P, PX, 256>), vh);
+  grid[2] = resident_grid(ctas_per_sm(bicg_update_p<P, 256>), vh);
+  grid[3] = resident_grid(ctas_per_sm(bicg_update_s<P, 256>), vh);
+  grid[4] = resident_grid(ctas_per_sm(bicg_update_xr<P, PX, 256>), vh);
 }
 
 struct Workspace {
