@@ -284,11 +284,11 @@ int wd_set_autotune(int enable);
  * for other sizes. */
 int wd_dslash_set_block(int sites);
 
-/* Launch overlap of consecutive single-field hopping kernels (the paper has
- * no such component).  enable = 1 (the default): every hopping launch of
- * wd_dslash, wd_dslash_dag, wd_dslash_ex, wd_mhat and the solvers, the
- * one-CTA launch that sums a fused norm's per-CTA partials, the CG and
- * BiCGstab vector updates of wd_solve_ex, wd_norm2, wd_cdot and wd_axpby are
+/* Launch overlap of consecutive kernels (the paper has no such component).
+ * enable = 1 (the default): the launches of wd_dslash, wd_dslash_dag,
+ * wd_dslash_ex, wd_mhat, wd_dslash_mrhs, wd_norm2, wd_cdot and wd_axpby, and
+ * those of the solvers' iterations where it pays (not in the captured
+ * iterations of small lattices, of FP64 and of wd_solve_batch), are
  * programmatic dependent launches.  The kernel first lets the next kernel of
  * the stream be scheduled once all of its own CTAs have started, then waits
  * until the previous kernel of the stream has completed and its writes are

@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(SUM_BS) sum_partials_kernel(const __grid_const
                                                               const double* __restrict__ partials,
                                                               double* out) {
   __shared__ double red[SUM_BS / 32];
+  pdl_begin();
   const int gi = blockIdx.x;
   int j = -1;
   for (int k = 0; k < L.nprob; k++)
@@ -87,8 +88,8 @@ static cudaError_t sum_partials(const B& bt, int units_per_tile, const int* acti
     nr = bt.p[j].rhs0 + bt.p[j].nrhs > nr ? bt.p[j].rhs0 + bt.p[j].nrhs : nr;
   }
   if (nr < 1) return cudaSuccess;
-  sum_partials_kernel<<<nr, SUM_BS, 0, st>>>(L, active, partials, out);
-  return cudaGetLastError();
+  return launch_with(!bt.plain, sum_partials_kernel, dim3(nr), dim3(SUM_BS), st, L, active,
+                     partials, out);
 }
 
 static cudaError_t launch_mrhs_raw(int prec, const MrhsBatch& bt, int recon, bool dagger,
@@ -330,36 +331,52 @@ struct BlasProblem {
   size_t s[3];
 };
 
-struct BlasBatch {
+template <int NP>
+struct BlasBatchOf {
+  static constexpr int problems = NP;
   int nprob, ntiles;
-  BlasProblem p[MRHS_MAX_PROBLEMS];
+  int plain;  // as in MrhsBatchOf
+  BlasProblem p[NP];
 };
+using BlasBatch = BlasBatchOf<MRHS_MAX_PROBLEMS>;
 
 #define WD_TILE_LOOP                                                   \
   for (int tile = blockIdx.x; tile < bt.ntiles; tile += gridDim.x) {   \
-    int j = 0;                                                         \
-    while (j + 1 < bt.nprob && tile >= bt.p[j + 1].tile0) j++;         \
-    const BlasProblem& pr = bt.p[j];                                   \
+    const BlasProblem& pr = bt.p[batch_problem(bt, tile)];             \
     const int cb = (tile - pr.tile0) * MRHS_BS + threadIdx.x;          \
     const bool valid = cb < pr.g.Vh;                                   \
     const int VP = pr.g.Vh_pad;
 
+// The quotients num / den of all active right-hand sides of the batch, once
+// per CTA (per thread and right-hand side the FP64 divisions of an update
+// took half as long as its memory traffic).  Ends with a barrier.
+template <typename T, typename B>
+__device__ __forceinline__ void batch_quotients(T* q, const B& bt, const int* active,
+                                                const double* num, const double* den) {
+  const BlasProblem& last = bt.p[bt.nprob - 1];
+  for (int gi = threadIdx.x; gi < last.rhs0 + last.nrhs; gi += MRHS_BS)
+    if (active[gi] != 0) q[gi] = (T)(num[gi] / den[gi]);
+  __syncthreads();
+}
+
 // r -= alpha q (f0 = r, f1 = q); alpha = gk / qq per rhs; per-(rhs, tile)
-// partials of ||r||^2, summed into rr by sum_partials_kernel
-template <int P>
-__global__ void __launch_bounds__(MRHS_BS) batch_update_r(const __grid_constant__ BlasBatch bt, const int* active,
-                                                          const double* gk, const double* qq,
-                                                          RedScratch rs, double* rr) {
+// partials of ||r||^2, summed by sum_partials_kernel
+template <int P, int NP>
+__global__ void __launch_bounds__(MRHS_BS)
+    batch_update_r(const __grid_constant__ BlasBatchOf<NP> bt, const int* active,
+                   const double* gk, const double* qq, RedScratch rs) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
-  (void)rr;
   __shared__ R red[MRHS_BS / 32];
+  __shared__ R sa[NP * MRHS_MAX];
+  pdl_begin();
+  batch_quotients(sa, bt, active, gk, qq);
   WD_TILE_LOOP
   for (int r = 0; r < pr.nrhs; r++) {
     const int gi = pr.rhs0 + r;
     if (active[gi] == 0) continue;
     R t = (R)0;
     if (valid) {
-      const R alpha = (R)(gk[gi] / qq[gi]);
+      const R alpha = sa[gi];
       char* fr = pr.f[0] + r * pr.s[0];
       const char* fq = pr.f[1] + r * pr.s[1];
       cx<R> a[12], b[12];
@@ -381,19 +398,24 @@ __global__ void __launch_bounds__(MRHS_BS) batch_update_r(const __grid_constant_
 }
 
 // x += alpha p ; p = s + beta p   (f0 = x [PX], f1 = p, f2 = s)
-template <int P, int PX>
-__global__ void __launch_bounds__(MRHS_BS) batch_update_xp(const __grid_constant__ BlasBatch bt, const int* active,
-                                                           const double* gk, const double* gk1,
-                                                           const double* qq) {
+template <int P, int PX, int NP>
+__global__ void __launch_bounds__(MRHS_BS)
+    batch_update_xp(const __grid_constant__ BlasBatchOf<NP> bt, const int* active,
+                    const double* gk, const double* gk1, const double* qq) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
   using RX = typename std::conditional<PX == WD_F64, double, float>::type;
+  __shared__ RX sa[NP * MRHS_MAX];
+  __shared__ R sb[NP * MRHS_MAX];
+  pdl_begin();
+  batch_quotients(sa, bt, active, gk, qq);
+  batch_quotients(sb, bt, active, gk1, gk);
   WD_TILE_LOOP
   if (!valid) continue;
   for (int r = 0; r < pr.nrhs; r++) {
     const int gi = pr.rhs0 + r;
     if (active[gi] == 0) continue;
-    const RX alpha = (RX)(gk[gi] / qq[gi]);
-    const R beta = (R)(gk1[gi] / gk[gi]);
+    const RX alpha = sa[gi];
+    const R beta = sb[gi];
     char* fx = pr.f[0] + r * pr.s[0];
     char* fp = pr.f[1] + r * pr.s[1];
     const char* fs = pr.f[2] + r * pr.s[2];
@@ -554,13 +576,6 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* b, long limit) {
   }
   __syncthreads();
   return ok_s != 0;
-}
-
-template <typename B>
-__device__ __forceinline__ int batch_problem(const B& bt, int tile) {
-  int j = 0;
-  while (j + 1 < bt.nprob && tile >= bt.p[j + 1].tile0) j++;
-  return j;
 }
 
 // The work items of a phase are (32-site sub-tile, right-hand side slot
@@ -900,8 +915,11 @@ void build_plan(BatchCtx& c, Plan& pl) {
   int nt = 0;
   for (auto& w : c.pw) nt = w.tile0 + w.ntiles;
   pl.ntiles = nt;
-  for (MrhsBatch* m : ms) { m->nprob = np; m->ntiles = nt; }
-  for (BlasBatch* b : bs) { b->nprob = np; b->ntiles = nt; }
+  // plain launches: in the captured iteration launch overlap gains nothing on
+  // large batches (12 right-hand sides on 16^3x32, FP32: 329 us an iteration
+  // either way) and costs up to a third on small ones (8^3x16: 86 against 65)
+  for (MrhsBatch* m : ms) { m->nprob = np; m->ntiles = nt; m->plain = 1; }
+  for (BlasBatch* b : bs) { b->nprob = np; b->ntiles = nt; b->plain = 1; }
   for (int j = 0; j < np; j++) {
     BatchProblemWs& w = c.pw[j];
     const double k = w.kappa, k2 = k * k;
@@ -945,15 +963,21 @@ cudaError_t batch_iteration_t(BatchCtx& c, const Plan& pl, int kp, cudaStream_t 
   c.dslash_calls += 4;
   if ((e = launch_mrhs(c.sprec, pl.d_oe_p, c.srecon, false, c.active, rs, nullptr, st))) return e;
   if ((e = launch_mrhs(c.sprec, pl.d_eo_q, c.srecon, false, c.active, rs, sc.qq, st))) return e;
-  batch_update_r<P><<<grid, MRHS_BS, 0, st>>>(pl.upd_r, c.active, sc.gamma[kp], sc.qq, rs, sc.rr);
-  if ((e = cudaGetLastError())) return e;
+  e = with_batch(pl.upd_r, [&](const auto& b) {
+    constexpr int NP = std::decay<decltype(b)>::type::problems;
+    return launch_with(!b.plain, batch_update_r<P, NP>, dim3(grid), dim3(MRHS_BS), st, b,
+                       c.active, sc.gamma[kp], sc.qq, rs);
+  });
+  if (e) return e;
   if ((e = sum_partials(pl.upd_r, 1, c.active, rs.partials, sc.rr, st))) return e;
   if ((e = launch_mrhs(c.sprec, pl.d_oe_r_dag, c.srecon, true, c.active, rs, nullptr, st))) return e;
   if ((e = launch_mrhs(c.sprec, pl.d_eo_s_dag, c.srecon, true, c.active, rs, sc.gamma[1 - kp], st)))
     return e;
-  batch_update_xp<P, PX><<<grid, MRHS_BS, 0, st>>>(pl.upd_xp, c.active, sc.gamma[kp],
-                                                   sc.gamma[1 - kp], sc.qq);
-  return cudaGetLastError();
+  return with_batch(pl.upd_xp, [&](const auto& b) {
+    constexpr int NP = std::decay<decltype(b)>::type::problems;
+    return launch_with(!b.plain, batch_update_xp<P, PX, NP>, dim3(grid), dim3(MRHS_BS), st, b,
+                       c.active, sc.gamma[kp], sc.gamma[1 - kp], sc.qq);
+  });
 }
 
 cudaError_t batch_iteration(BatchCtx& c, const Plan& pl, int kp, cudaStream_t st) {

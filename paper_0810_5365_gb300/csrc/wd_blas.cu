@@ -113,19 +113,20 @@ __global__ void __launch_bounds__(256) sum_blocks_kernel(const double* __restric
 }
 
 cudaError_t sum_block_partials(int n, const double* partials, int nblocks, SumOut out,
-                               cudaStream_t st) {
+                               cudaStream_t st, bool plain) {
+  const dim3 g(1), b(256);
   switch (n) {
-    case 1: return launch_pdl(sum_blocks_kernel<1>, dim3(1), dim3(256), st, partials, nblocks, out);
-    case 2: return launch_pdl(sum_blocks_kernel<2>, dim3(1), dim3(256), st, partials, nblocks, out);
-    case 3: return launch_pdl(sum_blocks_kernel<3>, dim3(1), dim3(256), st, partials, nblocks, out);
+    case 1: return launch_with(!plain, sum_blocks_kernel<1>, g, b, st, partials, nblocks, out);
+    case 2: return launch_with(!plain, sum_blocks_kernel<2>, g, b, st, partials, nblocks, out);
+    case 3: return launch_with(!plain, sum_blocks_kernel<3>, g, b, st, partials, nblocks, out);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t sum_block_partials(int n, const double* partials, int nblocks, double* out,
-                               cudaStream_t st) {
+                               cudaStream_t st, bool plain) {
   SumOut o = {{out, n > 1 ? out + 1 : nullptr, n > 2 ? out + 2 : nullptr}};
-  return sum_block_partials(n, partials, nblocks, o, st);
+  return sum_block_partials(n, partials, nblocks, o, st, plain);
 }
 
 RedScratch scratch() {

@@ -762,10 +762,10 @@ __global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>
   if constexpr (RED != RED_NONE) block_partials<NRED, BS>(red, a.rs.partials);
 }
 
-// Launch a hopping kernel (see launch_pdl)
+// Launch a hopping kernel (see launch_with)
 inline cudaError_t launch_hopping(void (*k)(const DslashArgs), dim3 grid, dim3 block,
                                   const DslashArgs& a, cudaStream_t st) {
-  return launch_pdl(k, grid, block, st, a);
+  return launch_with(!a.plain, k, grid, block, st, a);
 }
 
 // the non-reducing kernel with BS sites per CTA (64, 128 or 256)
@@ -819,7 +819,7 @@ cudaError_t launch_dslash_red_tg(const DslashArgs& a, dim3 grid, dim3 block, int
   cudaError_t e = launch_dslash_red_one<P, RC, DG, TG>(a, grid, block, bs, st);
   if (e != cudaSuccess || !a.norm_out || a.red_mode == RED_NONE) return e;
   const int nred = a.red_mode == RED_NORM ? 1 : a.red_mode == RED_NORM_DOTX ? 3 : 2;
-  return sum_block_partials(nred, a.rs.partials, (int)grid.x, a.norm_out, st);
+  return sum_block_partials(nred, a.rs.partials, (int)grid.x, a.norm_out, st, a.plain);
 }
 
 template <int P, int RC, bool DG>

@@ -240,8 +240,9 @@ cudaError_t launch_dslash_f16_staged(const DslashArgs& a, int recon, bool dagger
     cudaGetLastError();
     g_carveout_set[dev] = true;
   }
-  if (dagger) return launch_pdl(dslash_f16_staged_kernel<true>, grid, block, st, a, spin_limit);
-  return launch_pdl(dslash_f16_staged_kernel<false>, grid, block, st, a, spin_limit);
+  if (dagger)
+    return launch_with(!a.plain, dslash_f16_staged_kernel<true>, grid, block, st, a, spin_limit);
+  return launch_with(!a.plain, dslash_f16_staged_kernel<false>, grid, block, st, a, spin_limit);
 }
 
 // Read and clear the current device's fault flag after the work queued on

@@ -60,6 +60,8 @@ struct DslashArgs {
   const void* z = nullptr;
   // 1: never time launch shapes for this call (it must not allocate)
   int no_tune = 0;
+  // 1: plain stream-ordered launches (see launch_with)
+  int plain = 0;
 };
 
 // the run-time tuners (wd_batch.cu): on/off switch, a forced CTA size of the
@@ -71,12 +73,12 @@ void dslash_tune_record(const char* line);
 int launch_overlap();
 int set_launch_overlap(int enable);
 
-// Launch kernel k (which starts with pdl_begin) with launch overlap on
-// (wd_set_launch_overlap) as a programmatic dependent launch, else as a
-// plain stream-ordered launch.
+// Launch kernel k (which starts with pdl_begin) as a programmatic dependent
+// launch when `overlap` and launch overlap is on (wd_set_launch_overlap), else
+// as a plain stream-ordered launch.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
-                       Args... args) {
+cudaError_t launch_with(bool overlap, void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
+                        Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -86,8 +88,13 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t 
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = launch_overlap() ? 1 : 0;
+  cfg.numAttrs = overlap && launch_overlap() ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, args...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
+                       Args... args) {
+  return launch_with(true, k, grid, block, st, args...);
 }
 
 enum { RED_NONE = 0, RED_NORM = 1, RED_NORM_DOTX = 2, RED_DOTZ = 3 };
@@ -155,9 +162,9 @@ struct SumOut {
   double* p[3];
 };
 cudaError_t sum_block_partials(int n, const double* partials, int nblocks, SumOut out,
-                               cudaStream_t st);
+                               cudaStream_t st, bool plain = false);
 cudaError_t sum_block_partials(int n, const double* partials, int nblocks, double* out,
-                               cudaStream_t st);
+                               cudaStream_t st, bool plain = false);
 int num_sms();
 
 // grid of the grid-stride BLAS/reduction kernels for n sites

@@ -52,18 +52,22 @@ __host__ __device__ __forceinline__ void zdiv(double ar, double ai, double br, d
 }
 
 // The CG vector updates (and BiCGstab's p and s updates below) stream a few
-// fields once, about 10-20 us per call on 24^3x48.  They run on a grid of resident CTAs only (update_grid)
-// and each thread loads its next site before it computes the current one,
-// so that the load latency is paid about once per thread instead of once
-// per CTA generation.
+// fields once, about 10-20 us per call on 24^3x48.  Their scalars (quotients of
+// FP64 sums) are computed by one warp of a CTA and shared, behind the first
+// loads: a division is about ten FP64 instructions, each of which holds a
+// scheduler's FP64 pipe for 64 cycles, so with every warp computing its own
+// the eight warps of a scheduler took 2.7 us per division before any update.
+// They run on a grid of resident CTAs only (resident_grid) and each thread
+// loads its next site before it computes the current one, so that the load
+// latency is paid about once per thread instead of once per CTA generation.
 
 // r -= alpha q ; rr = ||r||^2 ; alpha = gamma[kp] / qq
 template <int P, int BS>
 __global__ void __launch_bounds__(BS) cg_update_r(char* r, const char* __restrict__ q,
                                                   CgScalars* sc, int kp, Geom g, RedScratch rs) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
+  __shared__ R sa;
   pdl_begin();
-  const R alpha = (R)(sc->gamma[kp] / sc->qq);
   R acc[1] = {(R)0};
   const int stride = gridDim.x * BS, VP = g.Vh_pad;
   int cb = blockIdx.x * BS + threadIdx.x;
@@ -72,6 +76,9 @@ __global__ void __launch_bounds__(BS) cg_update_r(char* r, const char* __restric
     load_raw<P>(ra, r, cb, VP);
     load_raw<P>(rb, q, cb, VP);
   }
+  if (threadIdx.x == 0) sa = (R)(sc->gamma[kp] / sc->qq);
+  __syncthreads();
+  const R alpha = sa;
   for (; cb < g.Vh; cb += stride) {
     const int nx = cb + stride;
     RawSite<P> na, nb;
@@ -102,10 +109,9 @@ __global__ void __launch_bounds__(BS, (P == WD_F16 ? 2 : 1))
                  Geom g) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
   using RX = typename std::conditional<PX == WD_F64, double, float>::type;
+  __shared__ RX sa;
+  __shared__ R sb;
   pdl_begin();
-  const double g0 = sc->gamma[kp];
-  const RX alpha = (RX)(g0 / sc->qq);
-  const R beta = (R)(sc->gamma[1 - kp] / g0);
   const int stride = gridDim.x * BS, VP = g.Vh_pad;
   int cb = blockIdx.x * BS + threadIdx.x;
   RawSite<P> rp, rsv;
@@ -115,6 +121,12 @@ __global__ void __launch_bounds__(BS, (P == WD_F16 ? 2 : 1))
     load_raw<P>(rsv, s, cb, VP);
     load_raw<PX>(rx, x, cb, VP);
   }
+  // (two warps: the divisions go to two schedulers)
+  if (threadIdx.x == 0) sa = (RX)(sc->gamma[kp] / sc->qq);
+  if (threadIdx.x == 32) sb = (R)(sc->gamma[1 - kp] / sc->gamma[kp]);
+  __syncthreads();
+  const RX alpha = sa;
+  const R beta = sb;
   for (; cb < g.Vh; cb += stride) {
     const int nx = cb + stride;
     RawSite<P> np, ns;
@@ -177,16 +189,8 @@ __global__ void __launch_bounds__(BS) bicg_update_p(char* p, const char* __restr
                                                     const char* __restrict__ v,
                                                     const CgScalars* sc, int kp, Geom g) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
+  __shared__ R sh[4];
   pdl_begin();
-  const int kq = 1 - kp;
-  double ar, ai, wr, wi, t1r, t1i, t2r, t2i, br, bi;
-  zdiv(sc->rho[kq][0], sc->rho[kq][1], sc->rv[kq][0], sc->rv[kq][1], ar, ai);   // alpha_old
-  zdiv(sc->tts[kq][1], sc->tts[kq][2], sc->tts[kq][0], 0.0, wr, wi);          // omega_old
-  zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rho[kq][0], sc->rho[kq][1], t1r, t1i);
-  zdiv(ar, ai, wr, wi, t2r, t2i);
-  br = t1r * t2r - t1i * t2i;
-  bi = t1r * t2i + t1i * t2r;
-  const R Br = (R)br, Bi = (R)bi, Wr = (R)wr, Wi = (R)wi;
   // resident grid, next site's loads first (as in cg_update_xp)
   const int stride = gridDim.x * BS, VP = g.Vh_pad;
   int cb = blockIdx.x * BS + threadIdx.x;
@@ -196,6 +200,20 @@ __global__ void __launch_bounds__(BS) bicg_update_p(char* p, const char* __restr
     load_raw<P>(rr, r, cb, VP);
     load_raw<P>(rv, v, cb, VP);
   }
+  if (threadIdx.x == 0) {
+    const int kq = 1 - kp;
+    double ar, ai, wr, wi, t1r, t1i, t2r, t2i;
+    zdiv(sc->rho[kq][0], sc->rho[kq][1], sc->rv[kq][0], sc->rv[kq][1], ar, ai);   // alpha_old
+    zdiv(sc->tts[kq][1], sc->tts[kq][2], sc->tts[kq][0], 0.0, wr, wi);          // omega_old
+    zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rho[kq][0], sc->rho[kq][1], t1r, t1i);
+    zdiv(ar, ai, wr, wi, t2r, t2i);
+    sh[0] = (R)(t1r * t2r - t1i * t2i);
+    sh[1] = (R)(t1r * t2i + t1i * t2r);
+    sh[2] = (R)wr;
+    sh[3] = (R)wi;
+  }
+  __syncthreads();
+  const R Br = sh[0], Bi = sh[1], Wr = sh[2], Wi = sh[3];
   for (; cb < g.Vh; cb += stride) {
     const int nx = cb + stride;
     RawSite<P> np, nr, nv;
@@ -229,10 +247,8 @@ __global__ void __launch_bounds__(BS) bicg_update_s(char* s, const char* __restr
                                                     const char* __restrict__ v,
                                                     const CgScalars* sc, int kp, Geom g) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
+  __shared__ R sh[2];
   pdl_begin();
-  double ar, ai;
-  zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rv[kp][0], sc->rv[kp][1], ar, ai);
-  const R Ar = (R)ar, Ai = (R)ai;
   // resident grid, next site's loads first (as in cg_update_r)
   const int stride = gridDim.x * BS, VP = g.Vh_pad;
   int cb = blockIdx.x * BS + threadIdx.x;
@@ -241,6 +257,14 @@ __global__ void __launch_bounds__(BS) bicg_update_s(char* s, const char* __restr
     load_raw<P>(rr, r, cb, VP);
     load_raw<P>(rv, v, cb, VP);
   }
+  if (threadIdx.x == 0) {
+    double ar, ai;
+    zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rv[kp][0], sc->rv[kp][1], ar, ai);
+    sh[0] = (R)ar;
+    sh[1] = (R)ai;
+  }
+  __syncthreads();
+  const R Ar = sh[0], Ai = sh[1];
   for (; cb < g.Vh; cb += stride) {
     const int nx = cb + stride;
     RawSite<P> nr, nv;
@@ -271,12 +295,17 @@ __global__ void __launch_bounds__(BS) bicg_update_xr(char* x, char* r, const cha
                                                      int kp, Geom g, RedScratch rs) {
   using R = typename std::conditional<P == WD_F64, double, float>::type;
   using RX = typename std::conditional<PX == WD_F64, double, float>::type;
+  __shared__ double sh[4];
   pdl_begin();
-  double ar, ai, wr, wi;
-  zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rv[kp][0], sc->rv[kp][1], ar, ai);
-  zdiv(sc->tts[kp][1], sc->tts[kp][2], sc->tts[kp][0], 0.0, wr, wi);
-  const RX Ar = (RX)ar, Ai = (RX)ai, Wxr = (RX)wr, Wxi = (RX)wi;
-  const R Wr = (R)wr, Wi = (R)wi;
+  // (no loads first: five fields of two sites leave no registers across the
+  // barrier; the two quotients go to two schedulers)
+  if (threadIdx.x == 0)
+    zdiv(sc->rho[kp][0], sc->rho[kp][1], sc->rv[kp][0], sc->rv[kp][1], sh[0], sh[1]);
+  if (threadIdx.x == 32)
+    zdiv(sc->tts[kp][1], sc->tts[kp][2], sc->tts[kp][0], 0.0, sh[2], sh[3]);
+  __syncthreads();
+  const RX Ar = (RX)sh[0], Ai = (RX)sh[1], Wxr = (RX)sh[2], Wxi = (RX)sh[3];
+  const R Wr = (R)sh[2], Wi = (R)sh[3];
   R acc[3] = {(R)0, (R)0, (R)0};
   if constexpr (P == WD_F64) {
     // (FP64: five prefetched sites do not fit the register file; plain loop)
@@ -532,8 +561,25 @@ struct Ctx {
   int sprec, srecon, orecon, xprec;
   int tg = 0;
   int bicg = 0;
+  int plain = 0;  // 1: plain stream-ordered launches (set while the graph is captured)
   double dslash_calls = 0;
 };
+
+// Launch overlap in the captured iteration pays where the hopping launches
+// fill the SMs: the next kernel's CTAs then start as the last wave drains.  On
+// lattices whose launches fit in one wave with room to spare the early CTAs
+// only get in the way, and a plain graph edge is the faster one.  us per CG
+// iteration, overlapped / plain: FP16 8^3x16 27 / 26, 16^4 38 / 28, 16^3x32
+// 42 / 37, 16^3x48 45 / 47, 24^3x48 116 / 118; FP32 16^3x32 50 / 42, 16^3x48
+// 58 / 55, 24^3x16 60 / 60, 24^3x48 180 / 182.  So: from 4/5 of a wave of
+// 128-site CTAs.  FP64 iterations gain nowhere (8^3x16 125 / 118, 32^3x64
+// 2798 / 2794) and are never overlapped.
+static bool graph_overlap(int prec, int vh) {
+  if (prec == WD_F64) return false;
+  const int per_sm =
+      prec == WD_F32 ? DslashMinBlocks<WD_F32, false>::value : DslashMinBlocks<WD_F16, false>::value;
+  return 5LL * ((vh + DSLASH_BS - 1) / DSLASH_BS) >= 4LL * per_sm * num_sms();
+}
 
 cudaError_t dsl(Ctx& c, int prec, int recon, const void* gauge, void* out, const void* in,
                 int parity, int dagger, double a, const void* x, double bx, const void* y,
@@ -555,6 +601,7 @@ cudaError_t dsl(Ctx& c, int prec, int recon, const void* gauge, void* out, const
   d.tg = c.tg;
   d.red_mode = red_mode;
   d.z = z;
+  d.plain = c.plain;
   c.dslash_calls += 1;
   return launch_dslash(prec, d, recon, dagger != 0, st);
 }
@@ -576,13 +623,13 @@ cudaError_t iteration_t(Ctx& c, int kp, cudaStream_t st) {
   const Geom& g = w.g;
   cudaError_t e = mhat_sloppy(c, w.q, w.p, 0, &w.sc->qq, st);
   if (e != cudaSuccess) return e;
-  if ((e = launch_pdl(cg_update_r<P, 256>, dim3(w.upd_grid[0]), dim3(256), st, (char*)w.r,
+  if ((e = launch_with(!c.plain, cg_update_r<P, 256>, dim3(w.upd_grid[0]), dim3(256), st, (char*)w.r,
                       (const char*)w.q, w.sc, kp, g, scratch())))
     return e;
-  if ((e = sum_block_partials(1, scratch().partials, w.upd_grid[0], &w.sc->rr, st))) return e;
+  if ((e = sum_block_partials(1, scratch().partials, w.upd_grid[0], &w.sc->rr, st, c.plain))) return e;
   e = mhat_sloppy(c, w.s, w.r, 1, &w.sc->gamma[1 - kp], st);
   if (e != cudaSuccess) return e;
-  return launch_pdl(cg_update_xp<P, PX, 256>, dim3(w.upd_grid[1]), dim3(256), st, (char*)w.xs,
+  return launch_with(!c.plain, cg_update_xp<P, PX, 256>, dim3(w.upd_grid[1]), dim3(256), st, (char*)w.xs,
                     (char*)w.p, (const char*)w.s, (const CgScalars*)w.sc, kp, g);
 }
 
@@ -593,7 +640,7 @@ cudaError_t iteration_bicg_t(Ctx& c, int kp, cudaStream_t st) {
   const Geom& g = w.g;
   const double k2 = c.kappa * c.kappa;
   cudaError_t e;
-  if ((e = launch_pdl(bicg_update_p<P, 256>, dim3(w.upd_grid[2]), dim3(256), st, (char*)w.p,
+  if ((e = launch_with(!c.plain, bicg_update_p<P, 256>, dim3(w.upd_grid[2]), dim3(256), st, (char*)w.p,
                       (const char*)w.r, (const char*)w.q, (const CgScalars*)w.sc, kp, g)))
     return e;
   // v = A p with <r0, v>
@@ -603,7 +650,7 @@ cudaError_t iteration_bicg_t(Ctx& c, int kp, cudaStream_t st) {
   if ((e = dsl(c, c.sprec, c.srecon, w.gs, w.q, w.ts, WD_EVEN, 0, -k2, w.p, 1.0, nullptr, 0,
                &w.sc->rv[kp][0], st, RED_DOTZ, w.r0)))
     return e;
-  if ((e = launch_pdl(bicg_update_s<P, 256>, dim3(w.upd_grid[3]), dim3(256), st, (char*)w.s,
+  if ((e = launch_with(!c.plain, bicg_update_s<P, 256>, dim3(w.upd_grid[3]), dim3(256), st, (char*)w.s,
                       (const char*)w.r, (const char*)w.q, (const CgScalars*)w.sc, kp, g)))
     return e;
   // t = A s with ||t||^2, <t, s>
@@ -613,12 +660,12 @@ cudaError_t iteration_bicg_t(Ctx& c, int kp, cudaStream_t st) {
   if ((e = dsl(c, c.sprec, c.srecon, w.gs, w.t, w.ts, WD_EVEN, 0, -k2, w.s, 1.0, nullptr, 0,
                &w.sc->tts[kp][0], st, RED_NORM_DOTX)))
     return e;
-  if ((e = launch_pdl(bicg_update_xr<P, PX, 256>, dim3(w.upd_grid[4]), dim3(256), st,
+  if ((e = launch_with(!c.plain, bicg_update_xr<P, PX, 256>, dim3(w.upd_grid[4]), dim3(256), st,
                       (char*)w.xs, (char*)w.r, (const char*)w.p, (const char*)w.s,
                       (const char*)w.t, (const char*)w.r0, w.sc, kp, g, scratch())))
     return e;
   SumOut o = {{&w.sc->rho[1 - kp][0], &w.sc->rho[1 - kp][1], &w.sc->rr}};
-  return sum_block_partials(3, scratch().partials, w.upd_grid[4], o, st);
+  return sum_block_partials(3, scratch().partials, w.upd_grid[4], o, st, c.plain);
 }
 
 cudaError_t iteration(Ctx& c, int kp, cudaStream_t st) {
@@ -801,7 +848,9 @@ int solve_impl(double* x, const double* b, const double* gauge, double kappa, co
     cudaGraph_t graph = nullptr;
     WD_CK(cudaStreamBeginCapture(w.cap, cudaStreamCaptureModeThreadLocal));
     cudaError_t ce = cudaSuccess;
+    c.plain = !graph_overlap(P.inner_prec, g.Vh);
     for (int k = 0; k < chunk && ce == cudaSuccess; k++) ce = iteration(c, k & 1, w.cap);
+    c.plain = 0;
     cudaError_t ee = cudaStreamEndCapture(w.cap, &graph);
     if (ce != cudaSuccess || ee != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
