@@ -31,6 +31,17 @@ int num_sms() {
   return s.num_sms;
 }
 
+size_t l2_bytes() {
+  State& s = state();
+  if (s.l2_bytes == 0) {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrL2CacheSize, dev);
+    s.l2_bytes = n > 0 ? (size_t)n : 1;
+  }
+  return s.l2_bytes;
+}
+
 int blas_grid(long long n, int bs) {
   long long need = (n + bs - 1) / bs;
   long long cap = (long long)num_sms() * (2048 / bs);

@@ -217,6 +217,31 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;\n" ::: "memory");
 }
 
+// Bring bytes (a multiple of 16, at a 16-byte boundary) into L2; nothing waits
+// for it.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p), "r"(bytes) : "memory");
+}
+
+// The FP16 links of directions mu < nmu that the n output sites from c0 on
+// (parity p) will read, brought into L2 by the first 4 nmu lanes of a warp, one
+// region and part each.  Backward links are taken at the shifted sites without
+// the wrap at the lattice's edge.  n and c0 even, c0 + n <= Vh.
+__device__ __forceinline__ void prefetch_links_f16(const void* gauge, const Geom& g, int p, int c0,
+                                                   int n, int nmu, int lane) {
+  if (lane >= 4 * nmu) return;
+  const int r = lane >> 1, mu = r >> 1;
+  const bool bwd = r & 1;
+  const int shift = !bwd || mu == 0 ? 0 : mu == 1 ? g.S1 : mu == 2 ? g.S2 : g.S3;
+  const int s = (c0 > shift ? c0 - shift : 0) & ~1;  // (8-byte part: 16-byte boundary)
+  const size_t at = (size_t)(2 * mu + (bwd ? 1 - p : p)) * g.Vh_pad + s;
+  const char* b = (const char*)gauge;
+  if (lane & 1)
+    prefetch_l2(b + (size_t)8 * g.Vh_pad * 16 + at * 8, n * 8);
+  else
+    prefetch_l2(b + at * 16, n * 16);
+}
+
 // A load of an input field.  COH = false: the read-only data path (the field
 // is not written while the kernel runs).  COH = true: an ordinary coherent
 // load, for a kernel that reads fields written earlier in the same launch by

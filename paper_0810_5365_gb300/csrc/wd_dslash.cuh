@@ -661,6 +661,11 @@ __global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>
   pdl_begin();
   const Geom& g = a.g;
   const int cb = blockIdx.x * BS + threadIdx.x;
+  if constexpr (P == WD_F16) {
+    const int c0 = blockIdx.x * BS + a.ahead;
+    if (a.ahead && threadIdx.x < 32 && c0 + BS <= g.Vh)
+      prefetch_links_f16(a.gauge, g, a.parity, c0, BS, TG ? 3 : 4, threadIdx.x);
+  }
   R red[NRED];
 #pragma unroll
   for (int j = 0; j < NRED; j++) red[j] = (R)0;
@@ -829,10 +834,23 @@ cudaError_t launch_dslash_red(const DslashArgs& a, dim3 grid, dim3 block, int bs
               : launch_dslash_red_tg<P, RC, DG, false>(a, grid, block, bs, st);
 }
 
+// How far ahead of its own sites an FP16 CTA brings links into L2.  The FP16
+// kernel is bound by the latency of its loads (HBM busy 0.85 of the time) and
+// the links are what it reads only once: half a microsecond of lead, by whole
+// 2 KB pieces, is worth 4 to 8 % where the links come from HBM.  us per launch
+// without / with: 32^3x64 54.8 / 52.5, with a fused norm 64.3 / 61.4, 48^3x64
+// 173.9 / 160.3.  1024 to 8192 sites of lead are the same to 0.5 %; a wave of
+// CTAs (117,000) gives 63 on 32^3x64.  Where the field's links fit in L2 it
+// only costs instructions (24^3x48: 18.2 / 18.6), so the line is at the
+// L2's size.  The kernel with staged neighbours loses (54.9 / 60.9).
+constexpr int F16_AHEAD = 4096;
+
 template <int P>
-cudaError_t launch_dslash_bs(const DslashArgs& a, int recon, bool dagger, int bs,
+cudaError_t launch_dslash_bs(const DslashArgs& args, int recon, bool dagger, int bs,
                              cudaStream_t st) {
   const int BS = DSLASH_BS;
+  DslashArgs a = args;
+  a.ahead = P == WD_F16 && gauge_bytes(a.g, WD_F16, 12) > l2_bytes() ? F16_AHEAD : 0;
   dim3 grid((a.g.Vh + BS - 1) / BS), block(BS);
   if (recon == 12)
     return dagger ? launch_dslash_red<P, 12, true>(a, grid, block, bs, st)

@@ -62,6 +62,9 @@ struct DslashArgs {
   int no_tune = 0;
   // 1: plain stream-ordered launches (see launch_with)
   int plain = 0;
+  // sites ahead of its own whose FP16 links a CTA brings into L2 (0: none);
+  // set by launch_dslash_bs
+  int ahead = 0;
 };
 
 // the run-time tuners (wd_batch.cu): on/off switch, a forced CTA size of the
@@ -140,6 +143,7 @@ struct State {
   unsigned* counter = nullptr;
   size_t partials_cap = 0;  // doubles
   int num_sms = 0;
+  size_t l2_bytes = 0;
   int* dev_flag = nullptr;  // device int: set by kernels whose bounded waits gave up
   // fields between the layers of wd_nn_apply*, partials of wd_nn_wgrad
   void* nn_scratch = nullptr;
@@ -166,6 +170,7 @@ cudaError_t sum_block_partials(int n, const double* partials, int nblocks, SumOu
 cudaError_t sum_block_partials(int n, const double* partials, int nblocks, double* out,
                                cudaStream_t st, bool plain = false);
 int num_sms();
+size_t l2_bytes();  // of the current device at the first call
 
 // grid of the grid-stride BLAS/reduction kernels for n sites
 int blas_grid(long long n, int bs);
