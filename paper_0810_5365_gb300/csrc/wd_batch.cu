@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(SUM_BS) sum_partials_kernel(const __grid_const
                                                               const int* active,
                                                               const double* __restrict__ partials,
                                                               double* out) {
-  __shared__ double red[SUM_BS / 32];
+  __shared__ double red[1][SUM_BS];
   pdl_begin();
   const int gi = blockIdx.x;
   int j = -1;
@@ -56,19 +56,10 @@ __global__ void __launch_bounds__(SUM_BS) sum_partials_kernel(const __grid_const
   if (j < 0 || (active != nullptr && active[gi] == 0)) return;  // uniform per block
   const int r = gi - L.rhs0[j];
   const double* row = partials + (size_t)r * L.stride + L.s0[j];
-  // four independent chains per thread keep four loads in flight; they are
-  // combined in a fixed order
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int t = threadIdx.x;
-  for (; t + 3 * SUM_BS < L.n[j]; t += 4 * SUM_BS) {
-    a0 += __ldcg(row + t);
-    a1 += __ldcg(row + t + SUM_BS);
-    a2 += __ldcg(row + t + 2 * SUM_BS);
-    a3 += __ldcg(row + t + 3 * SUM_BS);
-  }
-  for (; t < L.n[j]; t += SUM_BS) a0 += __ldcg(row + t);
-  double v[1] = {(a0 + a1) + (a2 + a3)};
-  block_sum<1, SUM_BS>(v, red);
+  // loads first, then as few FP64 additions as there are (see sum_blocks_kernel)
+  double v[1];
+  sum_strided<1, SUM_BS>(v, row, L.n[j], 1);
+  sum_threads<1, SUM_BS>(v, red);
   if (threadIdx.x == 0) out[gi] = v[0];
 }
 

@@ -81,41 +81,24 @@ cudaError_t device_flag(int** flag, cudaStream_t st) {
   return cudaMemsetAsync(s.dev_flag, 0, sizeof(int), st);
 }
 
-// The cross-block step of block_partials, in the same fixed order as the
-// last block of grid_reduce: CH chains per thread over the partials, combined
-// in order, then a block sum.
+// The cross-block step of block_partials: one CTA, a fixed order.  FP64
+// additions bound it: each of a warp holds its scheduler for 64 cycles, and
+// the two warps of a scheduler take turns.  So the partials are loaded first,
+// a thread adds only what it holds (sum_strided), and the threads' sums
+// meet through shared memory (one addition per halving, by half of the warps)
+// before the last warp's tree.  2592 partials: 26 additions on a scheduler's
+// path, where zero-initialised chains and a tree in every warp took 54; CG
+// iteration (three such sums), FP16: 24^3x48 115.5 -> 111.8 us, 16^3x32 38.0 ->
+// 35.2, 8^4 26.9 -> 24.7.
 template <int N>
 __global__ void __launch_bounds__(256) sum_blocks_kernel(const double* __restrict__ partials,
                                                          int nblocks, SumOut out) {
   constexpr int BS = 256;
-  constexpr int CH = N == 1 ? 8 : 4;
-  __shared__ double smem[N * (BS / 32)];
+  __shared__ double smem[N][BS];
   pdl_begin();
-  double part[CH][N];
-#pragma unroll
-  for (int c = 0; c < CH; c++)
-#pragma unroll
-    for (int j = 0; j < N; j++) part[c][j] = 0.0;
-  int b = threadIdx.x;
-  for (; b + (CH - 1) * BS < nblocks; b += CH * BS) {
-#pragma unroll
-    for (int c = 0; c < CH; c++)
-#pragma unroll
-      for (int j = 0; j < N; j++) part[c][j] += __ldcg(partials + (size_t)(b + c * BS) * N + j);
-  }
-  for (; b < nblocks; b += BS) {
-#pragma unroll
-    for (int j = 0; j < N; j++) part[0][j] += __ldcg(partials + (size_t)b * N + j);
-  }
   double acc[N];
-#pragma unroll
-  for (int j = 0; j < N; j++) {
-    double t = part[0][j];
-#pragma unroll
-    for (int c = 1; c < CH; c++) t += part[c][j];
-    acc[j] = t;
-  }
-  block_sum<N, BS>(acc, smem);
+  sum_strided<N, BS>(acc, partials, nblocks, N);
+  sum_threads<N, BS>(acc, smem);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int j = 0; j < N; j++)
@@ -433,8 +416,8 @@ cudaError_t convert_spinor(void* dst, int dprec, const void* src, int sprec, con
 // one addition per site, and the block tree once per thread, which with a
 // thread per site was most of the time (GB300's FP64 rate is 1/64 of FP32's).
 // They overlap their launch with the previous kernel's end (pdl_begin).
-// us per call on 24^3x48, FP32: norm2 13.0 -> 9.4, cdot 20.6 -> 11.6, axpby 10.3
-// -> 8.5; on 8^4 7.3 -> 5.3, 8.4 -> 6.8, 4.6 -> 4.3.
+// us per call on 24^3x48, FP32: norm2 13.1 -> 7.7, cdot 20.6 -> 9.5, axpby 10.3
+// -> 7.7; on 8^4 7.0 -> 4.6, 8.4 -> 5.9, 4.5 -> 4.3.
 
 // site i of nh halves
 template <int P>
@@ -459,6 +442,7 @@ __global__ void __launch_bounds__(RED_BS) norm2_kernel(double* res, const char* 
   for (; i < n; i += step) {
     RawSite<P> na;
     if (i + step < n) load_site<P>(na, x, i + step, g, hb);
+    asm volatile("" ::: "memory");  // the next site's loads are issued here
     cx<R> s[12];
     unpack_raw<P, R>(s, a);
     acc[0] += site_norm2(s);
@@ -488,6 +472,7 @@ __global__ void __launch_bounds__(RED_BS) cdot_kernel(double* res, const char* _
       load_site<P>(na, x, i + step, g, hb);
       load_site<P>(nb, y, i + step, g, hb);
     }
+    asm volatile("" ::: "memory");
     cx<R> u[12], v[12];
     unpack_raw<P, R>(u, a);
     unpack_raw<P, R>(v, b);
@@ -503,8 +488,9 @@ __global__ void __launch_bounds__(RED_BS) cdot_kernel(double* res, const char* _
 }
 
 template <int P>
-__global__ void __launch_bounds__(RED_BS) axpby_kernel(double a, const char* x, double b, char* y,
-                                                       Geom g, int nh, size_t hb) {
+__global__ void __launch_bounds__(RED_BS) axpby_kernel(double a, const char* __restrict__ x,
+                                                       double b, char* y, Geom g, int nh,
+                                                       size_t hb) {
   using R = real_of<P>;
   pdl_begin();
   const long long n = (long long)nh * g.Vh, step = (long long)gridDim.x * RED_BS;
@@ -512,26 +498,8 @@ __global__ void __launch_bounds__(RED_BS) axpby_kernel(double a, const char* x, 
   // b = 0: y is output only and never read (BLAS convention), so an
   // uninitialised y cannot leak NaN or Inf through 0 * y
   const bool read_y = b != 0.0;
-  // (FP64 sites are not loaded ahead: two sites of two fields take 210
-  // registers, and 45 instead of 35 us on 24^3x48, where the FP64 pipe bounds it)
-  constexpr bool AHEAD = P != WD_F64;
-  long long i = blockIdx.x * (long long)RED_BS + threadIdx.x;
-  RawSite<P> p, q, np, nq;
-  auto load = [&](RawSite<P>& o, RawSite<P>& w, long long at) {
-    if (at >= n) return;
-    load_site<P>(o, x, at, g, hb);
-    if (read_y) load_site<P>(w, y, at, g, hb);
-  };
-  if (AHEAD) load(p, q, i);
-  for (; i < n; i += step) {
-    if (AHEAD)
-      load(np, nq, i + step);
-    else
-      load(p, q, i);
-    cx<R> u[12], v[12];
-    unpack_raw<P, R>(u, p);
+  auto update = [&](cx<R>(&u)[12], cx<R>(&v)[12]) {
     if (read_y) {
-      unpack_raw<P, R>(v, q);
 #pragma unroll
       for (int k = 0; k < 12; k++) {
         v[k].r = ra * u[k].r + rb * v[k].r;
@@ -541,12 +509,55 @@ __global__ void __launch_bounds__(RED_BS) axpby_kernel(double a, const char* x, 
 #pragma unroll
       for (int k = 0; k < 12; k++) v[k] = mk<R>(ra * u[k].r, ra * u[k].i);
     }
+  };
+  long long i = blockIdx.x * (long long)RED_BS + threadIdx.x;
+  RawSite<P> p, q;
+  if (i < n) {
+    load_site<P>(p, x, i, g, hb);
+    if (read_y) load_site<P>(q, y, i, g, hb);
+  }
+  for (; i < n; i += step) {
+    RawSite<P> np, nq;
+    if (i + step < n) {
+      load_site<P>(np, x, i + step, g, hb);
+      if (read_y) load_site<P>(nq, y, i + step, g, hb);
+    }
+    cx<R> u[12], v[12];
+    unpack_raw<P, R>(u, p);
+    if (read_y) unpack_raw<P, R>(v, q);
+    update(u, v);
     const bool odd = i >= g.Vh;
     store_spinor<P, R>(odd ? y + hb : y, (int)(odd ? i - g.Vh : i), g.Vh_pad, v);
-    if (AHEAD) {
-      p = np;
-      q = nq;
+    p = np;
+    q = nq;
+  }
+}
+
+// FP64 axpby: bound by the FP64 pipe, and fastest with the site's elements
+// loaded as they are used (34 registers, eight CTAs per SM): loading ahead
+// takes 210 registers and 45 us on 24^3x48, a site at a time 106 and 39,
+// against 35.  It does not overlap its launch: the next grid's CTAs then crowd
+// on the SMs that have room (16^3x32: 22 us against 10).
+__global__ void axpby_f64_kernel(double a, const char* __restrict__ x, double b, char* y, Geom g,
+                                 int nh, size_t hb) {
+  const long long n = (long long)nh * g.Vh;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int h = (int)(i / g.Vh), cb = (int)(i - (long long)h * g.Vh);
+    cx<double> u[12], v[12];
+    load_spinor_rw<WD_F64, double>(u, x + h * hb, cb, g.Vh_pad);
+    if (b != 0.0) {
+      load_spinor_rw<WD_F64, double>(v, y + h * hb, cb, g.Vh_pad);
+#pragma unroll
+      for (int k = 0; k < 12; k++) {
+        v[k].r = a * u[k].r + b * v[k].r;
+        v[k].i = a * u[k].i + b * v[k].i;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 12; k++) v[k] = mk<double>(a * u[k].r, a * u[k].i);
     }
+    store_spinor<WD_F64, double>(y + h * hb, cb, g.Vh_pad, v);
   }
 }
 
@@ -556,8 +567,10 @@ static cudaError_t norm2_p(double* res, const void* x, const Geom& g, int nh, cu
   const int grid = resident_grid(per_sm, (long long)nh * g.Vh);
   cudaError_t e = ensure_scratch((size_t)grid * 2);
   if (e != cudaSuccess) return e;
-  return launch_pdl(norm2_kernel<P>, dim3(grid), dim3(RED_BS), st, res, (const char*)x, g, nh,
-                    spinor_half_bytes(g, P), scratch());
+  // (FP64 on a part-filled GPU: 11.5 us overlapped, 10.4 plain on 16^3x32)
+  return launch_with(P != WD_F64 || grid == per_sm * num_sms(), norm2_kernel<P>, dim3(grid),
+                     dim3(RED_BS), st, res, (const char*)x, g, nh, spinor_half_bytes(g, P),
+                     scratch());
 }
 template <int P>
 static cudaError_t cdot_p(double* res, const void* x, const void* y, const Geom& g, int nh,
@@ -600,7 +613,10 @@ cudaError_t cdot(double* res, const void* x, const void* y, const Geom& g, int p
 cudaError_t axpby(double a, const void* x, double b, void* y, const Geom& g, int prec, int nh,
                   cudaStream_t st) {
   switch (prec) {
-    case WD_F64: return axpby_p<WD_F64>(a, x, b, y, g, nh, st);
+    case WD_F64:
+      axpby_f64_kernel<<<blas_grid((long long)nh * g.Vh, 256), 256, 0, st>>>(
+          a, (const char*)x, b, (char*)y, g, nh, spinor_half_bytes(g, WD_F64));
+      return cudaGetLastError();
     case WD_F32: return axpby_p<WD_F32>(a, x, b, y, g, nh, st);
     case WD_F16: return axpby_p<WD_F16>(a, x, b, y, g, nh, st);
     default: return cudaErrorInvalidValue;

@@ -657,6 +657,76 @@ __device__ __forceinline__ void block_sum(T (&v)[N], T* smem /* N * BS/32 */) {
   }
 }
 
+// Sum over the BS threads of a block in FP64, in a fixed order, with few
+// additions per scheduler: halves of the block are folded through shared
+// memory until one warp is left.  The total is in thread 0.
+template <int N, int BS>
+__device__ __forceinline__ void sum_threads(double (&v)[N], double (*smem)[BS]) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int half = BS / 2; half >= 32; half /= 2) {
+    if (tid >= half && tid < 2 * half) {
+#pragma unroll
+      for (int j = 0; j < N; j++) smem[j][tid] = v[j];
+    }
+    __syncthreads();
+    if (tid < half) {
+#pragma unroll
+      for (int j = 0; j < N; j++) v[j] += smem[j][tid + half];
+    }
+  }
+  if (tid < 32) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < N; j++) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+  }
+}
+
+// v[j] = sum over k < n of p[k stride + j], this thread's k = threadIdx.x + i BS,
+// loaded twelve at a time before they are added.  (A jump into the additions,
+// not a condition on each: an FP64 addition that is predicated off still takes
+// its 64 cycles.)
+template <int N, int BS>
+__device__ __forceinline__ void sum_strided(double (&v)[N], const double* __restrict__ p, int n,
+                                            int stride) {
+#pragma unroll
+  for (int j = 0; j < N; j++) v[j] = 0.0;
+  for (int k0 = threadIdx.x; k0 < n; k0 += 12 * BS) {
+    double w[12][N];
+#pragma unroll
+    for (int c = 0; c < 12; c++)
+#pragma unroll
+      for (int j = 0; j < N; j++)
+        if (k0 + c * BS < n) w[c][j] = __ldcg(p + (size_t)(k0 + c * BS) * stride + j);
+    auto add = [&](int c) {
+#pragma unroll
+      for (int j = 0; j < N; j++) v[j] += w[c][j];
+    };
+    const int here = (n - k0 + BS - 1) / BS;
+    if (k0 < BS) {
+#pragma unroll
+      for (int j = 0; j < N; j++) v[j] = w[0][j];
+    } else {
+      add(0);
+    }
+    switch (here < 12 ? here : 12) {
+      case 12: add(11); [[fallthrough]];
+      case 11: add(10); [[fallthrough]];
+      case 10: add(9); [[fallthrough]];
+      case 9: add(8); [[fallthrough]];
+      case 8: add(7); [[fallthrough]];
+      case 7: add(6); [[fallthrough]];
+      case 6: add(5); [[fallthrough]];
+      case 5: add(4); [[fallthrough]];
+      case 4: add(3); [[fallthrough]];
+      case 3: add(2); [[fallthrough]];
+      case 2: add(1); [[fallthrough]];
+      default: break;
+    }
+  }
+}
+
 // The block's share of a grid sum, without the cross-block step: the block
 // sums v in T and thread 0 stores its N totals as FP64 partials.  A separate
 // launch that follows the kernel in its stream (sum_block_partials) adds the
@@ -673,14 +743,18 @@ __device__ __forceinline__ void block_partials(T (&v)[N], double* partials) {
 }
 
 // Returns true in every thread of the last block; there `tot` holds the grid
-// total in thread 0 (and all threads of warp 0).  The block sums in T (the
+// total in thread 0.  The block sums in T (the
 // kernel's working precision), the block partials in FP64.
 template <int N, int BS, typename T = double>
 __device__ __forceinline__ bool grid_reduce(T (&v)[N], RedScratch rs, double (&tot)[N]) {
-  __shared__ T tsmem[N * (BS / 32)];
-  __shared__ double smem[N * (BS / 32)];
+  // (more than four sums do not get a word per thread of shared memory)
+  constexpr bool FOLD = N <= 4;
+  __shared__ double smem[N][FOLD ? BS : BS / 32];
   __shared__ bool last;
-  block_sum<N, BS, T>(v, tsmem);
+  if constexpr (FOLD && std::is_same<T, double>::value)
+    sum_threads<N, BS>(v, smem);
+  else
+    block_sum<N, BS, T>(v, reinterpret_cast<T*>(smem));
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int j = 0; j < N; j++) rs.partials[(size_t)blockIdx.x * N + j] = (double)v[j];
@@ -694,36 +768,20 @@ __device__ __forceinline__ bool grid_reduce(T (&v)[N], RedScratch rs, double (&t
   __syncthreads();
   if (!last) return false;
   __threadfence();
-  // CH independent chains per thread keep CH loads of the partials in flight
-  // (a single chain waits one L2 round trip per partial); the chains are
-  // combined in a fixed order, so the sum does not depend on scheduling
-  constexpr int CH = N == 1 ? 8 : (N <= 4 ? 4 : 1);
-  double part[CH][N];
-#pragma unroll
-  for (int c = 0; c < CH; c++)
-#pragma unroll
-    for (int j = 0; j < N; j++) part[c][j] = 0.0;
-  int b = threadIdx.x;
-  for (; b + (CH - 1) * BS < (int)gridDim.x; b += CH * BS) {
-#pragma unroll
-    for (int c = 0; c < CH; c++)
-#pragma unroll
-      for (int j = 0; j < N; j++) part[c][j] += __ldcg(rs.partials + (size_t)(b + c * BS) * N + j);
-  }
-  for (; b < (int)gridDim.x; b += BS) {
-#pragma unroll
-    for (int j = 0; j < N; j++) part[0][j] += __ldcg(rs.partials + (size_t)b * N + j);
-  }
   double acc[N];
+  if constexpr (FOLD) {
+    sum_strided<N, BS>(acc, rs.partials, (int)gridDim.x, N);
+  } else {
 #pragma unroll
-  for (int j = 0; j < N; j++) {
-    double t = part[0][j];
+    for (int j = 0; j < N; j++) acc[j] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += BS)
 #pragma unroll
-    for (int c = 1; c < CH; c++) t += part[c][j];
-    acc[j] = t;
+      for (int j = 0; j < N; j++) acc[j] += __ldcg(rs.partials + (size_t)b * N + j);
   }
-  __syncthreads();
-  block_sum<N, BS>(acc, smem);
+  if constexpr (FOLD)
+    sum_threads<N, BS>(acc, smem);
+  else
+    block_sum<N, BS>(acc, &smem[0][0]);
 #pragma unroll
   for (int j = 0; j < N; j++) tot[j] = acc[j];
   if (threadIdx.x == 0) *rs.counter = 0u;
