@@ -281,12 +281,18 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
     fix_cross(U[6], U[1], U[5], U[2], U[4]);
     fix_cross(U[7], U[2], U[3], U[0], U[5]);
     fix_cross(U[8], U[0], U[4], U[1], U[3]);
-    // (rows that are not orthonormal can give a larger row 2)
+    // (rows that are not orthonormal can give a larger row 2, which the sums
+    // have no room for: t or 2 L - t is negative when |V.h| > L)
+    constexpr unsigned L = (1u << 27) + 128;
     unsigned big = 0;
 #pragma unroll
     for (int k = 6; k < 9; k++)
-      big |= ((unsigned)(U[k][0].h + (1 << 27) + 128) | (unsigned)(U[k][1].h + (1 << 27) + 128));
-    acc.bad |= big >> 29;
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const unsigned t = (unsigned)U[k][j].h + L;
+        big |= t | (2 * L - t);
+      }
+    acc.bad |= big >> 31;
   }
 #pragma unroll
   for (int c = 0; c < 3; c++) {

@@ -199,6 +199,19 @@ int main() {
       return 1;
     }
   }
+  // rows of ordinary size whose row 2 is larger (12-real storage, not SU(3))
+  for (double z : {1.0, 0.6, -0.6, -1.0}) {
+    double u[12] = {1, 0, 0, z, 0, 0, 0, z, 1, 0, 0, 0};  // row 2 = (0, 0, 1 + z^2)
+    FixSite s;
+    fix_begin(s);
+    cx<double> h[6];
+    for (auto& v : h) v = {gau(), gau()};
+    fix_hop<1, true, 12>(s, 0, h, u, false, false);
+    if (fix_ok(s)) {
+      printf("FAIL refusal of row 2 (%g)\n", z);
+      return 1;
+    }
+  }
   printf("OK %d %.3f\n", n, worst);
   return 0;
 }
