@@ -462,17 +462,14 @@ __device__ __forceinline__ void store_f16_h2(void* base, int cb, int Vh_pad,
   }
 }
 
-#ifndef WD_F16_PREFETCH
-#define WD_F16_PREFETCH 2
-#endif
-
 // The eight hops of one FP16 site: the eight neighbour scales are loaded
 // first, then the loads of the next hops are issued before the current one
-// is computed (WD_F16_PREFETCH hops in flight).  The hops are accumulated in
+// is computed (two hops in flight at the 80-register budget, three with
+// DEEP at 128 registers).  The hops are accumulated in
 // half2 relative to the largest neighbour scale (compute_f16), which is
 // returned: H in at this site = smax * ah.  funit/bunit: the
 // forward/backward time link is the identity (temporal gauge).
-template <int SF, int SB_, bool COH = false>
+template <int SF, int SB_, bool COH = false, bool DEEP = false>
 __device__ __forceinline__ float hops_f16(__half2 (&ah)[12], const void* __restrict__ in,
                                           const void* __restrict__ ga, int p, int cb, int f0,
                                           int b0, int f1, int b1, int f2, int b2, int f3, int b3,
@@ -485,61 +482,36 @@ __device__ __forceinline__ float hops_f16(__half2 (&ah)[12], const void* __restr
 #pragma unroll
   for (int k = 0; k < 12; k++) ah[k] = __float2half2_rn(0.f);
 #define WD_F(nb, reg, lcb) fetch_f16<COH>(in, ga, nb, reg, lcb, VP)
-#if WD_F16_PREFETCH >= 3
   RawF16 r0 = WD_F(f0, 0 + p, cb), r1 = WD_F(b0, 0 + q, b0);
-  RawF16 r2 = WD_F(f1, 2 + p, cb), r3 = WD_F(b1, 2 + q, b1);
+  RawF16 r2 = WD_F(f1, 2 + p, cb), r3;
+  if constexpr (DEEP) r3 = WD_F(b1, 2 + q, b1);
   __half2 rel[4];
   const float smax = f16_rel(sc, fflip, bflip, rel);
   compute_f16<0, SF, true>(ah, r0, __low2half2(rel[0]));
-  r0 = WD_F(f2, 4 + p, cb);
+  if constexpr (DEEP)
+    r0 = WD_F(f2, 4 + p, cb);
+  else
+    r3 = WD_F(b1, 2 + q, b1);
   compute_f16<0, SB_, false>(ah, r1, __high2half2(rel[0]));
-  r1 = WD_F(b2, 4 + q, b2);
+  if constexpr (DEEP)
+    r1 = WD_F(b2, 4 + q, b2);
+  else
+    r0 = WD_F(f2, 4 + p, cb);
   compute_f16<1, SF, true>(ah, r2, __low2half2(rel[1]));
-  r2 = fetch_f16<COH>(in, ga, f3, 6 + p, cb, VP, funit);
+  if constexpr (DEEP)
+    r2 = fetch_f16<COH>(in, ga, f3, 6 + p, cb, VP, funit);
+  else
+    r1 = WD_F(b2, 4 + q, b2);
   compute_f16<1, SB_, false>(ah, r3, __high2half2(rel[1]));
-  r3 = fetch_f16<COH>(in, ga, b3, 6 + q, b3, VP, bunit);
+  if constexpr (DEEP)
+    r3 = fetch_f16<COH>(in, ga, b3, 6 + q, b3, VP, bunit);
+  else
+    r2 = fetch_f16<COH>(in, ga, f3, 6 + p, cb, VP, funit);
   compute_f16<2, SF, true>(ah, r0, __low2half2(rel[2]));
+  if constexpr (!DEEP) r3 = fetch_f16<COH>(in, ga, b3, 6 + q, b3, VP, bunit);
   compute_f16<2, SB_, false>(ah, r1, __high2half2(rel[2]));
   compute_f16<3, SF, true>(ah, r2, __low2half2(rel[3]), funit);
   compute_f16<3, SB_, false>(ah, r3, __high2half2(rel[3]), bunit);
-#elif WD_F16_PREFETCH >= 2
-  RawF16 r0 = WD_F(f0, 0 + p, cb), r1 = WD_F(b0, 0 + q, b0);
-  RawF16 r2 = WD_F(f1, 2 + p, cb);
-  __half2 rel[4];
-  const float smax = f16_rel(sc, fflip, bflip, rel);
-  compute_f16<0, SF, true>(ah, r0, __low2half2(rel[0]));
-  RawF16 r3 = WD_F(b1, 2 + q, b1);
-  compute_f16<0, SB_, false>(ah, r1, __high2half2(rel[0]));
-  r0 = WD_F(f2, 4 + p, cb);
-  compute_f16<1, SF, true>(ah, r2, __low2half2(rel[1]));
-  r1 = WD_F(b2, 4 + q, b2);
-  compute_f16<1, SB_, false>(ah, r3, __high2half2(rel[1]));
-  r2 = fetch_f16<COH>(in, ga, f3, 6 + p, cb, VP, funit);
-  compute_f16<2, SF, true>(ah, r0, __low2half2(rel[2]));
-  r3 = fetch_f16<COH>(in, ga, b3, 6 + q, b3, VP, bunit);
-  compute_f16<2, SB_, false>(ah, r1, __high2half2(rel[2]));
-  compute_f16<3, SF, true>(ah, r2, __low2half2(rel[3]), funit);
-  compute_f16<3, SB_, false>(ah, r3, __high2half2(rel[3]), bunit);
-#else
-  RawF16 r0 = WD_F(f0, 0 + p, cb);
-  RawF16 r1 = WD_F(b0, 0 + q, b0);
-  __half2 rel[4];
-  const float smax = f16_rel(sc, fflip, bflip, rel);
-  compute_f16<0, SF, true>(ah, r0, __low2half2(rel[0]));
-  r0 = WD_F(f1, 2 + p, cb);
-  compute_f16<0, SB_, false>(ah, r1, __high2half2(rel[0]));
-  r1 = WD_F(b1, 2 + q, b1);
-  compute_f16<1, SF, true>(ah, r0, __low2half2(rel[1]));
-  r0 = WD_F(f2, 4 + p, cb);
-  compute_f16<1, SB_, false>(ah, r1, __high2half2(rel[1]));
-  r1 = WD_F(b2, 4 + q, b2);
-  compute_f16<2, SF, true>(ah, r0, __low2half2(rel[2]));
-  r0 = fetch_f16<COH>(in, ga, f3, 6 + p, cb, VP, funit);
-  compute_f16<2, SB_, false>(ah, r1, __high2half2(rel[2]));
-  r1 = fetch_f16<COH>(in, ga, b3, 6 + q, b3, VP, bunit);
-  compute_f16<3, SF, true>(ah, r0, __low2half2(rel[3]), funit);
-  compute_f16<3, SB_, false>(ah, r1, __high2half2(rel[3]), bunit);
-#endif
 #undef WD_F
   return smax;
 }
@@ -647,21 +619,38 @@ __device__ __forceinline__ void hops_f64(cx<double> (&acc)[12], const void* __re
 // its register budget)
 // BS sites per CTA; the register budget per thread is that of the 128-site
 // CTAs for every BS (the same number of resident warps)
-template <int P, bool NORM, int BS>
+//
+// DEEP (FP32 and FP16): the kernel for lattices all of whose CTAs are resident
+// at 128 registers.  There the time is one site's chain of loads and hops, not
+// bandwidth, and registers beyond the ordinary 72 to 80 are free: more of the
+// loads are in flight at once (FP32 by the compiler's own order, FP16 by three
+// hops ahead instead of two).  us per launch in a graph, ordinary / DEEP, FP32
+// and FP16: 8^4 3.54 / 2.91 and 3.19 / 2.77; 14x10x18x22 4.86 / 4.15 and 3.90
+// / 3.64; 16^4 4.56 / 4.00 and 3.73 / 3.49; 16^3x32 6.24 / 6.00 and 5.18 /
+// 4.92; with a fused norm 8^4 6.05 / 5.33 and 5.51 / 5.18, 16^3x32 8.57 / 8.40
+// and 7.75 / 7.55; in a stream with launch overlap, which also crowds fewer
+// CTAs of a grid on one SM at this budget, 16^4 FP32 8.5 / 5.8, M-hat FP16 on
+// 14x10x18x22 13.3 / 9.9.  Beyond one wave it loses (24^4 FP32 13.5 / 13.9, FP16 8.85
+// / 9.02), so the line is where its own wave ends (dslash_deep).  A budget of
+// 255 registers gives another 6 % on 8^4 and loses 9 % on 16^3x32.  Same
+// operations in the same order: the same bits.
+constexpr int DEEP_MINB = 4;
+
+template <int P, bool NORM, int BS, bool DEEP>
 struct DslashMinBlocksBS {
-  static constexpr int raw = DslashMinBlocks<P, NORM>::value * DSLASH_BS / BS;
+  static constexpr int raw = (DEEP ? DEEP_MINB : DslashMinBlocks<P, NORM>::value) * DSLASH_BS / BS;
   static constexpr int value = raw < 1 ? 1 : raw;
 };
 
-template <int P, int RC, bool DAG, int RED, bool TG, int BS>
-__global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>::value))
+template <int P, int RC, bool DAG, int RED, bool TG, int BS, bool DEEP>
+__global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS, DEEP>::value))
     dslash_kernel(const DslashArgs a) {
   constexpr int NRED = RED == RED_NONE ? 1 : RED == RED_NORM ? 1 : RED == RED_NORM_DOTX ? 3 : 2;
   using R = typename std::conditional<P == WD_F64, double, float>::type;
   pdl_begin();
   const Geom& g = a.g;
   const int cb = blockIdx.x * BS + threadIdx.x;
-  if constexpr (P == WD_F16) {
+  if constexpr (P == WD_F16 && !DEEP) {
     const int c0 = blockIdx.x * BS + a.ahead;
     if (a.ahead && threadIdx.x < 32 && c0 + BS <= g.Vh)
       prefetch_links_f16(a.gauge, g, a.parity, c0, BS, TG ? 3 : 4, threadIdx.x);
@@ -700,9 +689,9 @@ __global__ void __launch_bounds__(BS, (DslashMinBlocksBS<P, RED != RED_NONE, BS>
       constexpr int SF = DAG ? -1 : 1;
       constexpr int SB_ = -SF;
       __half2 ah[12];
-      const float kf = (float)a.a * hops_f16<SF, SB_>(ah, a.in, a.gauge, p, cb, f0, b0, f1, b1,
-                                                      f2, b2, f3, b3, fflip, bflip, funit, bunit,
-                                                      VP);
+      const float kf = (float)a.a * hops_f16<SF, SB_, false, DEEP>(ah, a.in, a.gauge, p, cb, f0,
+                                                                   b0, f1, b1, f2, b2, f3, b3,
+                                                                   fflip, bflip, funit, bunit, VP);
       if (!a.x && !a.y) {
         store_f16_h2<RED != RED_NONE>(a.out, cb, VP, ah, kf, acc);
         stored = true;
@@ -774,42 +763,42 @@ inline cudaError_t launch_hopping(void (*k)(const DslashArgs), dim3 grid, dim3 b
 }
 
 // the non-reducing kernel with BS sites per CTA (64, 128 or 256)
-template <int P, int RC, bool DG, bool TG>
+template <int P, int RC, bool DG, bool TG, bool DEEP>
 cudaError_t launch_dslash_plain_bs(const DslashArgs& a, int bs, cudaStream_t st) {
   const unsigned n = (unsigned)a.g.Vh;
   switch (bs) {
     case 64:
-      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, 64>, dim3((n + 63) / 64),
+      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, 64, DEEP>, dim3((n + 63) / 64),
                             dim3(64), a, st);
     case 256:
-      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, 256>, dim3((n + 255) / 256),
+      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, 256, DEEP>, dim3((n + 255) / 256),
                             dim3(256), a, st);
     default:
-      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, DSLASH_BS>,
+      return launch_hopping(dslash_kernel<P, RC, DG, RED_NONE, TG, DSLASH_BS, DEEP>,
                             dim3((n + DSLASH_BS - 1) / DSLASH_BS), dim3(DSLASH_BS), a, st);
   }
 }
 
-template <int P, int RC, bool DG, bool TG>
+template <int P, int RC, bool DG, bool TG, bool DEEP>
 cudaError_t launch_dslash_red_one(const DslashArgs& a, dim3 grid, dim3 block, int bs,
                                   cudaStream_t st) {
   const int mode = a.norm_out ? a.red_mode : RED_NONE;
   switch (mode) {
     case RED_NONE:
-      return launch_dslash_plain_bs<P, RC, DG, TG>(a, bs, st);
+      return launch_dslash_plain_bs<P, RC, DG, TG, DEEP>(a, bs, st);
     case RED_NORM:
-      return launch_hopping(dslash_kernel<P, RC, DG, RED_NORM, TG, DSLASH_BS>, grid, block, a, st);
+      return launch_hopping(dslash_kernel<P, RC, DG, RED_NORM, TG, DSLASH_BS, DEEP>, grid, block, a, st);
     case RED_NORM_DOTX:
     case RED_DOTZ:
       // the dot-product epilogues serve BiCGstab, which never applies H^+
       if constexpr (!DG) {
         if (mode == RED_NORM_DOTX) {
           if (!a.x) return cudaErrorInvalidValue;
-          return launch_hopping(dslash_kernel<P, RC, DG, RED_NORM_DOTX, TG, DSLASH_BS>, grid,
+          return launch_hopping(dslash_kernel<P, RC, DG, RED_NORM_DOTX, TG, DSLASH_BS, DEEP>, grid,
                                 block, a, st);
         }
         if (!a.z) return cudaErrorInvalidValue;
-        return launch_hopping(dslash_kernel<P, RC, DG, RED_DOTZ, TG, DSLASH_BS>, grid, block, a,
+        return launch_hopping(dslash_kernel<P, RC, DG, RED_DOTZ, TG, DSLASH_BS, DEEP>, grid, block, a,
                               st);
       }
       return cudaErrorInvalidValue;
@@ -817,11 +806,21 @@ cudaError_t launch_dslash_red_one(const DslashArgs& a, dim3 grid, dim3 block, in
   }
 }
 
+// whether the CTAs of one parity all fit on the SMs at the DEEP budget
+template <int P>
+bool dslash_deep(int vh) {
+  return P != WD_F64 && (vh + DSLASH_BS - 1) / DSLASH_BS <= DEEP_MINB * num_sms();
+}
+
 // a reducing launch is followed by the sum of its block partials
 template <int P, int RC, bool DG, bool TG>
 cudaError_t launch_dslash_red_tg(const DslashArgs& a, dim3 grid, dim3 block, int bs,
                                  cudaStream_t st) {
-  cudaError_t e = launch_dslash_red_one<P, RC, DG, TG>(a, grid, block, bs, st);
+  cudaError_t e;
+  if (dslash_deep<P>(a.g.Vh))
+    e = launch_dslash_red_one<P, RC, DG, TG, P != WD_F64>(a, grid, block, bs, st);
+  else
+    e = launch_dslash_red_one<P, RC, DG, TG, false>(a, grid, block, bs, st);
   if (e != cudaSuccess || !a.norm_out || a.red_mode == RED_NONE) return e;
   const int nred = a.red_mode == RED_NORM ? 1 : a.red_mode == RED_NORM_DOTX ? 3 : 2;
   return sum_block_partials(nred, a.rs.partials, (int)grid.x, a.norm_out, st, a.plain);
