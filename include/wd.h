@@ -288,12 +288,11 @@ int wd_dslash_set_block(int sites);
  * enable = 1 (the default): the launches of wd_dslash, wd_dslash_dag,
  * wd_dslash_ex, wd_mhat, wd_dslash_mrhs, wd_norm2, wd_cdot and wd_axpby, and
  * those of the solvers' iterations where it pays (not in the captured
- * iterations of small lattices, of FP64 and of wd_solve_batch, nor for FP64
- * axpby), are
- * programmatic dependent launches.  The kernel first lets the next kernel of
- * the stream be scheduled once all of its own CTAs have started, then waits
- * until the previous kernel of the stream has completed and its writes are
- * visible, before it reads or writes any memory.  So consecutive launches
+ * iterations of medium lattices, of FP64 and of wd_solve_batch, nor for FP64
+ * axpby), are programmatic dependent launches.  The kernel first waits until
+ * the previous kernel of the stream has completed and its writes are visible,
+ * before it reads or writes any memory, then lets the next kernel be scheduled
+ * once all of its own CTAs have got that far.  So consecutive launches
  * overlap only their scheduling (the next grid's CTAs take the SM slots that
  * the last wave frees), never their memory accesses, and results are
  * bit-identical with either setting.  enable = 0: plain stream-ordered

@@ -628,9 +628,7 @@ __device__ __forceinline__ void hops_f64(cx<double> (&acc)[12], const void* __re
 // and FP16: 8^4 3.54 / 2.91 and 3.19 / 2.77; 14x10x18x22 4.86 / 4.15 and 3.90
 // / 3.64; 16^4 4.56 / 4.00 and 3.73 / 3.49; 16^3x32 6.24 / 6.00 and 5.18 /
 // 4.92; with a fused norm 8^4 6.05 / 5.33 and 5.51 / 5.18, 16^3x32 8.57 / 8.40
-// and 7.75 / 7.55; in a stream with launch overlap, which also crowds fewer
-// CTAs of a grid on one SM at this budget, 16^4 FP32 8.5 / 5.8, M-hat FP16 on
-// 14x10x18x22 13.3 / 9.9.  Beyond one wave it loses (24^4 FP32 13.5 / 13.9, FP16 8.85
+// and 7.75 / 7.55.  Beyond one wave it loses (24^4 FP32 13.5 / 13.9, FP16 8.85
 // / 9.02), so the line is where its own wave ends (dslash_deep).  A budget of
 // 255 registers gives another 6 % on 8^4 and loses 9 % on 16^3x32.  Same
 // operations in the same order: the same bits.

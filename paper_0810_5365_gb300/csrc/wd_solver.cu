@@ -566,19 +566,22 @@ struct Ctx {
 };
 
 // Launch overlap in the captured iteration pays where the hopping launches
-// fill the SMs: the next kernel's CTAs then start as the last wave drains.  On
-// lattices whose launches fit in one wave with room to spare the early CTAs
-// only get in the way, and a plain graph edge is the faster one.  us per CG
-// iteration, overlapped / plain: FP16 8^3x16 27 / 26, 16^4 38 / 28, 16^3x32
-// 42 / 37, 16^3x48 45 / 47, 24^3x48 116 / 118; FP32 16^3x32 50 / 42, 16^3x48
-// 58 / 55, 24^3x16 60 / 60, 24^3x48 180 / 182.  So: from 4/5 of a wave of
-// 128-site CTAs.  FP64 iterations gain nowhere (8^3x16 125 / 118, 32^3x64
-// 2798 / 2794) and are never overlapped.
+// fill the SMs, so that the next kernel's CTAs start as the last wave drains,
+// and where they leave SMs empty.  In between the early CTAs get in the way,
+// and a plain graph edge is the faster one.  us per iteration, overlapped /
+// plain: FP16 CG 4^4 20.5 / 22.0, 8^3x16 22.0 / 23.2, 12^4 22.4 / 24.1, 12^3x24
+// 24.5 / 25.5, 16^3x24 31.8 / 31.4; FP32 CG 4^4 22.0 / 23.2, 8^3x16 23.2 / 24.5,
+// 12^4 25.4 / 24.8, 16^4 29.6 / 28.1, 24^3x12 49 / 45, 16^3x48 54.0 / 51.5;
+// BiCGstab like CG.  24^3x48 FP16 116 / 118, FP32 180 / 182.  So: from 4/5 of a
+// wave of 128-site CTAs, and up to one CTA per SM in FP16 and one per two SMs
+// in FP32.  FP64 iterations gain nowhere (4^4 114 / 111, 8^3x16 115 / 115, 16^3x24
+// 184 / 174, 24^3x20 442 / 441) and are never overlapped.
 static bool graph_overlap(int prec, int vh) {
   if (prec == WD_F64) return false;
   const int per_sm =
       prec == WD_F32 ? DslashMinBlocks<WD_F32, false>::value : DslashMinBlocks<WD_F16, false>::value;
-  return 5LL * ((vh + DSLASH_BS - 1) / DSLASH_BS) >= 4LL * per_sm * num_sms();
+  const int ctas = (vh + DSLASH_BS - 1) / DSLASH_BS;
+  return 5LL * ctas >= 4LL * per_sm * num_sms() || (prec == WD_F16 ? ctas : 2 * ctas) <= num_sms();
 }
 
 cudaError_t dsl(Ctx& c, int prec, int recon, const void* gauge, void* out, const void* in,
