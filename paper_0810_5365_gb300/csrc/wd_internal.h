@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "wd_common.cuh"
 
 namespace wd {
@@ -149,6 +151,7 @@ struct State {
   void* nn_scratch = nullptr;
   size_t nn_scratch_bytes = 0;
   int nn_scratch_dev = -1;
+  std::atomic<bool> nn_scratch_taken{false};
   // polls of the first bounded wait of the asynchronous kernels (wd_set_wait_limit)
   long wait_limit = 1L << 22;
 };

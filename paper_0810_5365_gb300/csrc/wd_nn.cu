@@ -913,22 +913,28 @@ struct Alloc {
 // Scratch of the synchronous network calls (wd_nn_apply*, wd_nn_wgrad): kept
 // between calls, since a cudaMalloc/cudaFree pair of its size costs as much as
 // the kernels (wd_nn_apply_ex on 32^3x64, BF16: 0.9 ms of kernels, 1.0 ms of
-// allocation).  Every call that uses it returns with its stream idle (after
-// an error too), so the next one may use it on another stream.  At most NN_SCRATCH_KEEP bytes stay
-// allocated (32^3x64 needs 0.8 GB); a larger lattice's are freed with the
-// call, and wd_finalize frees the rest.
+// allocation).  One call at a time has it: a call that finds it taken by
+// another host thread allocates its own.  Every call returns it with its
+// stream idle (after an error too), so the next one may use it on another
+// stream.  At most NN_SCRATCH_KEEP bytes stay allocated (32^3x64 needs 0.8 GB);
+// a larger lattice's are freed with the call, and wd_finalize frees the rest.
 constexpr size_t NN_SCRATCH_KEEP = (size_t)1 << 30;
 
 struct NnScratch {
   char* at = nullptr;
   bool idle = false;  // the call has synchronised its stream
-  Alloc own;          // a request above NN_SCRATCH_KEEP
+  bool held = false;  // the call has the kept scratch
+  cudaStream_t st = state().stream;
+  Alloc own;          // a request above NN_SCRATCH_KEEP, or the kept one taken
   ~NnScratch() {
-    if (!idle) cudaStreamSynchronize(state().stream);
+    if (!idle) cudaStreamSynchronize(st);
+    if (held) state().nn_scratch_taken.store(false);
   }
   cudaError_t get(size_t bytes) {
-    if (bytes > NN_SCRATCH_KEEP) return own.get((void**)&at, bytes);
     State& s = state();
+    if (bytes > NN_SCRATCH_KEEP || s.nn_scratch_taken.exchange(true))
+      return own.get((void**)&at, bytes);
+    held = true;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

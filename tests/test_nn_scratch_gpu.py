@@ -46,3 +46,30 @@ def test_network_calls_share_one_scratch():
     finally:
         W.wd_set_stream(None)
         W.wd_finalize()
+
+
+def test_two_host_threads_do_not_share_it():
+    import threading
+    import torch
+    import paper_0810_5365_gb300 as W
+    dims = (8, 8, 8, 8)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda n: torch.randn(n, device="cuda", generator=g)  # noqa: E731
+    gauge = (0.3 * rnd(W.wd_gauge_bytes(dims, W.WD_F32, 12) // 4)).view(torch.uint8)
+    work = [(0.2 * rnd(W.WD_NN_PARAMS), rnd(W.nn_field_bytes(dims, 4) // 4)) for _ in range(2)]
+
+    def apply(w, x):
+        o = torch.zeros_like(x)
+        W.wd_nn_apply_ex(o, x, w, gauge, dims, W.WD_NN_BF16)
+        return o
+
+    ref = [apply(*c) for c in work]
+    outs = [[], []]
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=lambda k=k: outs[k].extend(apply(*work[k]) for _ in range(100))) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in (0, 1):
+        assert len(outs[k]) == 100 and all(torch.equal(o, ref[k]) for o in outs[k])
