@@ -146,8 +146,11 @@ __host__ __device__ __forceinline__ void fix_begin(FixSite& acc) {
 
 // Raise the site's scale to that of the projected half spinor h when h is
 // larger (to one bit above it, so that few of the later hops raise it again:
-// each time costs the shift of all sums).  False: h vanishes, nothing to add.
-__host__ __device__ __forceinline__ bool fix_scale(FixSite& acc, const cx<double> (&h)[6]) {
+// each time costs the shift of all sums).  A half spinor that vanishes goes
+// through the products like any other: they come out as zero, a link that does
+// not fit is seen (0 times NaN is NaN), and the time of a launch, which the
+// tuners compare, does not depend on how much of a field is zero.
+__host__ __device__ __forceinline__ void fix_scale(FixSite& acc, const cx<double> (&h)[6]) {
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k < 6; k++) {
@@ -163,7 +166,6 @@ __host__ __device__ __forceinline__ bool fix_scale(FixSite& acc, const cx<double
 #pragma unroll
     for (int k = 0; k < 6; k++) lows |= d_bits(h[k].r) | d_bits(h[k].i);
     acc.bad |= (unsigned)lows;
-    return false;
   }
   const int e = (int)(m >> 20);
   if (e > acc.E) {
@@ -175,7 +177,6 @@ __host__ __device__ __forceinline__ bool fix_scale(FixSite& acc, const cx<double
       acc.i[k] >>= d;
     }
   }
-  return true;
 }
 
 // The largest |high word| of n link reals so far, and at the end whether the
@@ -248,7 +249,7 @@ __host__ __device__ __forceinline__ void fix_expand(FixSite& acc, int mu, int c,
 template <int S, bool FWD, int RC>
 __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<double> (&h)[6],
                                                  const double (&u)[RC], bool flip, bool unit) {
-  if (!fix_scale(acc, h)) return;
+  fix_scale(acc, h);
   Limb H[6][2];
 #pragma unroll
   for (int k = 0; k < 6; k++) {
