@@ -583,9 +583,9 @@ __device__ __forceinline__ void hop_fix(FixSite& fx, int mu, const void* __restr
 }
 
 // The eight hops of one FP64 site: fixed point, or the FP64 chain where the
-// values do not fit it.  24^3x48, one parity, us per launch: FP64 chain 541
-// (recon 18) and 788 (recon 12, which rebuilds row 2 on the FP64 pipe), fixed
-// point 175 and 196.  What bounds it now: the integer pipes (ALU 42 % busy)
+// values do not fit it.  24^3x48, one parity, us per launch: FP64 chain 537
+// (recon 18) and 686 (recon 12, which rebuilds row 2 on the FP64 pipe), fixed
+// point 185 and 212.  What bounds it now: the integer pipes (ALU 42 % busy)
 // through the latency of dependent instructions, with 12 warps per SM at 168
 // registers; 8 or 16 warps (255 registers, or 128 and spills) are slower.  The
 // directions are a loop, not unrolled: eight copies of the hop (200 KB of
@@ -606,7 +606,7 @@ __device__ __forceinline__ void hops_f64(cx<double> (&acc)[12], const void* __re
     hop_fix<RC, -SF, false, COH>(fx, mu, in, ga, b, 2 * mu + 1 - p, b, mu == 3 && nb.bflip, VP,
                                  mu == 3 && nb.bunit);
   }
-  if (fix_ok(fx)) {
+  if (fix_ok(fx) && fix_resolved(fx)) {
 #pragma unroll
     for (int k = 0; k < 12; k++)
       acc[k] = mk<double>(fix_double(fx.r[k], fx.E), fix_double(fx.i[k], fx.E));

@@ -8,28 +8,45 @@
 // stay on that pipe; the SU(3) product and the sum over the eight hops run on
 // integers.
 //
-// Formats (E: the site's scale, a biased exponent not below that of any
-// projected component seen so far, e = E - 1023):
-//   half spinor  h = H 2^(e-60), |H| < 2^61
-//   link         u = V 2^-59,    |V| < 2^59 (1 + 2^-20)
-//   sums         t = T 2^(e-55), below 2^62 after eight hops
+// Formats (E: the site's scale, a biased exponent, e = E - 1023; no projected
+// component seen so far is 1.5 2^e or more):
+//   half spinor  h = H 2^(e-61), |H| < 1.5 2^61
+//   link         u = V 2^-61,    |V| < 2^61 (1 + 2^-20)
+//   products     t = T 2^(e-58), below 2^60 each (fix_ok; rows of a norm of up
+//                to one cannot give more), so that the sum of eight fits 64 bits
 // H and V are cut into two signed 32-bit limbs, x = x.h 2^32 + x.l, and
 // H V = H.h V.h 2^64 + (H.h V.l + H.l V.h) 2^32 + H.l V.l.  The last product
-// is dropped (below 2^-56 of the largest |h|, rms), the middle ones are summed
+// is dropped (below 2^-59 of the largest |h|, rms), the middle ones are summed
 // and rounded once per component and hop.  The FP64 chain rounds each of
-// its 6 + 1 additions per hop at 2^-53 of the partial sum.  Errors relative to
-// the rms component of the site, both against 64-bit-mantissa references:
-// fixed point 0.58e-16, chain 1.42e-16 on Gaussian neighbours of one size; the
-// fixed-point one is the smaller for every form tried (unit links, single
-// colours, sizes spread over 2^+-40: tests/host/fix64_check.cu).
+// its 6 + 1 additions per hop at 2^-53 of the partial sum.
 //
-// A site falls back to the FP64 chain when a value does not fit: |u| above 1
-// or a link that is small throughout (not SU(3)), infinities, NaN, or
-// exponents near the ends of the range.
+// Error: a site's sums share one scale, so the fixed-point error, 2^-58 of it
+// (rms), is the same for all components, where the chain's goes with each
+// component's own products.  Against 64-bit mantissas, relative to the rms
+// component of the site: fixed point 0.48e-16, chain 1.42e-16 on Gaussian
+// neighbours of one size, and the smaller for every form tried (unit links,
+// single colours, sizes spread over 2^+-40: tests/host/fix64_check.cu).  A
+// component whose products stay below 2^-5 of the scale would get fewer bits
+// than the chain gives it (links that do not mix the colours, a spin that is
+// small): its site takes the chain (fix_resolved).  Component by component the
+// error is 0.41 of the chain's for products of one size and 0.95 of it at that
+// line (tests/host/fix64_small_check.cu; 2^-6 would be 1.5 times the chain's).
+//
+// A site also falls back to the FP64 chain when a value does not fit: |u| above
+// 1 or a link that is small throughout (not SU(3)), infinities, NaN, or
+// exponents near the ends of the range.  Where that happens the site costs both
+// (24^3x48, us, all sites in the chain / none: 660 / 185 with 18-real links,
+// 813 / 212 with 12).  On Gaussian fields and on solutions and residuals of
+// Gaussian sources no site does; on the propagator of a point source 0.1 to 2 %
+// of the warps hold one with links of mean 0.94 (216 to 230 us, 18-real), most
+// of them with smoother links (exp(0.15 i H): 410 to 560).
 //
 // Instructions per hop: 30 conversions of 11 (a 64-bit shift written on two
 // 32-bit words: on a 64-bit variable the compiler took 16), 216 multiply-adds,
-// about 100 for the sums and 60 for the scale.
+// about 150 for the sums and their sizes and 60 for the scale.  The sizes and
+// the three bits that T has for the line at 2^-5 (a carry between the halves of
+// a row) cost 6 to 9 %: 174 -> 185 us and, with 12-real links, 193 -> 212; at
+// 2^-3 without those bits the propagators above took the chain everywhere.
 #pragma once
 
 #include <string.h>
@@ -48,10 +65,22 @@ struct FixSite {
   int E;          // biased exponent of the scale
   unsigned any;   // non-zero: some neighbour was not zero
   unsigned bad;   // non-zero: a value did not fit
+  // how large the hops' products have been (fix_size): of the x and y hops, of
+  // the z and t hops, one word per colour, spin 0 in its low half
+  unsigned xy[3], zt[3];
 };
 
 constexpr int FIX_EMIN = 128;   // smallest and largest scale handled
 constexpr int FIX_EMAX = 1980;
+// A component is resolved when one of its products reaches 2^-5 of the scale:
+// fix_size's bits from T = 2^53 on.
+constexpr unsigned FIX_FINE = 0xffc0ffc0u;
+// Eight products below T = 2^60 cannot overflow: the bits from there on.
+constexpr unsigned FIX_FULL = 0xe000e000u;
+// The scale is one bit above the largest component's power of two where that
+// component is 1.5 times it or more: a row of norm one then gives less than
+// sqrt(6) 1.5 2^58 < 2^60.
+constexpr unsigned FIX_ROOM = 0x80000u;
 constexpr unsigned FIX_UMAX = 0x3ff00000u;  // high words of |u| < 1 + 2^-20 ...
 constexpr unsigned FIX_UMIN = 0x3fc00000u;  // ... and of 1/8 (an SU(3) row has a real >= 0.23)
 
@@ -103,7 +132,8 @@ __host__ __device__ __forceinline__ Limb fix_neg(Limb a) {
   return o;
 }
 
-// one real of a sum of products
+// One real of a sum of products, in two halves of at most four products each
+// (their middle terms add up to less than 2^63): fix_carry between them.
 struct FixAcc {
   long long A, B;
 };
@@ -111,6 +141,10 @@ __host__ __device__ __forceinline__ void fix_mac(FixAcc& s, Limb u, Limb h) {
   s.A += (long long)u.h * h.h;
   s.B += (long long)u.h * h.l;
   s.B += (long long)u.l * h.h;
+}
+__host__ __device__ __forceinline__ void fix_carry(FixAcc& s) {
+  s.A += s.B >> 32;
+  s.B = (long long)(unsigned)s.B;
 }
 __host__ __device__ __forceinline__ long long fix_round(const FixAcc& s) {
   return s.A + (s.B >> 32);
@@ -121,32 +155,41 @@ __host__ __device__ __forceinline__ void fix_cross(Limb (&o)[2], const Limb (&a)
                                                    const Limb (&b)[2], const Limb (&c)[2],
                                                    const Limb (&d)[2]) {
   const Limb nbi = fix_neg(b[1]), ndr = fix_neg(d[0]), nbr = fix_neg(b[0]);
-  FixAcc re = {0, 1LL << 26}, im = {0, 1LL << 26};
-  fix_mac(re, a[0], b[0]);
-  fix_mac(re, a[1], nbi);
-  fix_mac(re, c[0], ndr);
-  fix_mac(re, c[1], d[1]);
+  FixAcc re = {0, 1LL << 28}, im = {0, 1LL << 28};
   // -(a.r b.i + a.i b.r - c.r d.i - c.i d.r)
+  fix_mac(re, a[0], b[0]);
   fix_mac(im, a[0], nbi);
+  fix_mac(re, a[1], nbi);
   fix_mac(im, a[1], nbr);
+  fix_carry(re);
+  fix_carry(im);
+  fix_mac(re, c[0], ndr);
   fix_mac(im, c[0], d[1]);
+  fix_mac(re, c[1], d[1]);
   fix_mac(im, c[1], d[0]);
-  // products 2^-118 -> 2^-59
-  o[0] = fix_split(re.A * 32 + (re.B >> 27));
-  o[1] = fix_split(im.A * 32 + (im.B >> 27));
+  // products 2^-122 -> 2^-61 (up to 2^63 where |u| is up to one: fix_hop's check
+  // sees the wrapped value too)
+  o[0] = fix_split((long long)((unsigned long long)re.A * 8) + (re.B >> 29));
+  o[1] = fix_split((long long)((unsigned long long)im.A * 8) + (im.B >> 29));
 }
 
 // Site state before its first hop.
 __host__ __device__ __forceinline__ void fix_begin(FixSite& acc) {
 #pragma unroll
   for (int k = 0; k < 12; k++) acc.r[k] = acc.i[k] = 0;
+#pragma unroll
+  for (int c = 0; c < 3; c++) acc.xy[c] = acc.zt[c] = 0;
   acc.E = FIX_EMIN;
   acc.any = acc.bad = 0;
 }
 
+__host__ __device__ __forceinline__ unsigned fix_sizes(const FixSite& a) {
+  return a.xy[0] | a.xy[1] | a.xy[2] | a.zt[0] | a.zt[1] | a.zt[2];
+}
+
 // Raise the site's scale to that of the projected half spinor h when h is
-// larger (to one bit above it, so that few of the later hops raise it again:
-// each time costs the shift of all sums).  A half spinor that vanishes goes
+// larger (with some room, so that few of the later hops raise it again: each
+// time costs the shift of all sums).  A half spinor that vanishes goes
 // through the products like any other: they come out as zero, a link that does
 // not fit is seen (0 times NaN is NaN), and the time of a launch, which the
 // tuners compare, does not depend on how much of a field is zero.
@@ -167,14 +210,22 @@ __host__ __device__ __forceinline__ void fix_scale(FixSite& acc, const cx<double
     for (int k = 0; k < 6; k++) lows |= d_bits(h[k].r) | d_bits(h[k].i);
     acc.bad |= (unsigned)lows;
   }
-  const int e = (int)(m >> 20);
+  const int e = (int)((m + FIX_ROOM) >> 20);
   if (e > acc.E) {
-    const int d = e + 1 - acc.E < 63 ? e + 1 - acc.E : 63;
-    acc.E = e + 1;
+    const int d = e - acc.E < 63 ? e - acc.E : 63;
+    acc.E = e;
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       acc.r[k] >>= d;
       acc.i[k] >>= d;
+    }
+    const int dw = d < 16 ? d : 16;
+    const unsigned keep = (0xffffu >> dw) * 0x10001u;
+    acc.bad |= fix_sizes(acc) & FIX_FULL;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      acc.xy[c] = (acc.xy[c] >> dw) & keep;
+      acc.zt[c] = (acc.zt[c] >> dw) & keep;
     }
   }
 }
@@ -194,14 +245,34 @@ __host__ __device__ __forceinline__ void fix_row(long long& tr, long long& ti,
   FixAcc re = {0, 1LL << 31}, im = {0, 1LL << 31};
 #pragma unroll
   for (int d = 0; d < 3; d++) {
-    const Limb n = fix_neg(H[d][FWD ? 1 : 0]);
     fix_mac(re, v[d][0], H[d][0]);
-    fix_mac(re, v[d][1], FWD ? n : H[d][1]);
     fix_mac(im, v[d][0], H[d][1]);
+  }
+  fix_carry(re);
+  fix_carry(im);
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const Limb n = fix_neg(H[d][FWD ? 1 : 0]);
+    fix_mac(re, v[d][1], FWD ? n : H[d][1]);
     fix_mac(im, v[d][1], FWD ? H[d][0] : n);
   }
   tr = fix_round(re);
   ti = fix_round(im);
+}
+
+// The size of two products: the bits at which v's leading 16 differ from the
+// bit below, the first in the low half of the word, the second in the high one
+// (bit b + 1 of T is set where |T| >= 2^b; the carry from the low half only
+// reaches bit 0 of the high one)
+__host__ __device__ __forceinline__ unsigned fix_size(long long v0, long long v1) {
+  const unsigned a = (unsigned)((unsigned long long)v0 >> 32);
+  const unsigned b = (unsigned)((unsigned long long)v1 >> 32);
+#ifdef __CUDA_ARCH__
+  const unsigned w = __byte_perm(a, b, 0x7632);
+#else
+  const unsigned w = (a >> 16) | (b & 0xffff0000u);
+#endif
+  return w ^ (w << 1);
 }
 
 // Colour c of the expansion of expand_add: upper spins t0, t1, lower spins
@@ -209,6 +280,11 @@ __host__ __device__ __forceinline__ void fix_row(long long& tr, long long& ti,
 template <int S>
 __host__ __device__ __forceinline__ void fix_expand(FixSite& acc, int mu, int c, long long r0,
                                                     long long i0, long long r1, long long i1) {
+  const unsigned w = fix_size(r0, r1) | fix_size(i0, i1);
+  if (mu < 2)
+    acc.xy[c] |= w;
+  else
+    acc.zt[c] |= w;
   acc.r[c] += r0;
   acc.i[c] += i0;
   acc.r[3 + c] += r1;
@@ -253,8 +329,8 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
   Limb H[6][2];
 #pragma unroll
   for (int k = 0; k < 6; k++) {
-    H[k][0] = fix_limbs(d_bits(h[k].r), acc.E + 3);
-    H[k][1] = fix_limbs(d_bits(h[k].i), acc.E + 3);
+    H[k][0] = fix_limbs(d_bits(h[k].r), acc.E + 2);
+    H[k][1] = fix_limbs(d_bits(h[k].i), acc.E + 2);
   }
   if (flip) {
 #pragma unroll
@@ -266,7 +342,7 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
   if (unit) {
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      auto t = [](Limb a) { return ((((long long)a.h << 32) + a.l) + 16) >> 5; };
+      auto t = [](Limb a) { return ((((long long)a.h << 32) + a.l) + 4) >> 3; };
       fix_expand<S>(acc, mu, c, t(H[c][0]), t(H[c][1]), t(H[3 + c][0]), t(H[3 + c][1]));
     }
     return;
@@ -277,14 +353,14 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
 #pragma unroll
     for (int k = 0; k < RC; k++) {
       fix_link_max(um, d_bits(u[k]));
-      U[k >> 1][k & 1] = fix_limbs(d_bits(u[k]), 1023 + 4);
+      U[k >> 1][k & 1] = fix_limbs(d_bits(u[k]), 1023 + 2);
     }
     fix_cross(U[6], U[1], U[5], U[2], U[4]);
     fix_cross(U[7], U[2], U[3], U[0], U[5]);
     fix_cross(U[8], U[0], U[4], U[1], U[3]);
     // (rows that are not orthonormal can give a larger row 2, which the sums
     // have no room for: t or 2 L - t is negative when |V.h| > L)
-    constexpr unsigned L = (1u << 27) + 128;
+    constexpr unsigned L = (1u << 29) + 512;
     unsigned big = 0;
 #pragma unroll
     for (int k = 6; k < 9; k++)
@@ -307,7 +383,7 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
           v[d][j] = U[k][j];
         } else {
           fix_link_max(um, d_bits(u[2 * k + j]));
-          v[d][j] = fix_limbs(d_bits(u[2 * k + j]), 1023 + 4);
+          v[d][j] = fix_limbs(d_bits(u[2 * k + j]), 1023 + 2);
         }
       }
     }
@@ -321,10 +397,29 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
 
 // whether the site's sums are valid (else: the FP64 chain)
 __host__ __device__ __forceinline__ bool fix_ok(const FixSite& a) {
-  return a.bad == 0 && a.E < FIX_EMAX && (a.E > FIX_EMIN || a.any == 0);
+  return (a.bad | (fix_sizes(a) & FIX_FULL)) == 0 && a.E < FIX_EMAX && (a.E > FIX_EMIN || a.any == 0);
 }
 
-// T 2^(E - 1023 - 55) as a double, rounded to nearest
+// Whether every component of the site has as many bits as the FP64 chain would
+// give it.  The sums of a site share one scale, so a component all of whose
+// products are small keeps fewer bits (none, 2^-55 below the scale), where the
+// chain rounds each relative to its own products.  With links that mix the
+// colours the products of a component are of the size of its neighbours; with
+// links that do not (unit, diagonal) a colour can stay small.  Spins 0 and 1
+// add the products of their own rows; spins 2 and 3 those of spins 1 and 0
+// along x and y, of 0 and 1 along z and t.
+__host__ __device__ __forceinline__ bool fix_resolved(const FixSite& a) {
+  bool all = true;
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    const unsigned up = (a.xy[c] | a.zt[c]) & FIX_FINE;
+    const unsigned low = (((a.xy[c] << 16) | (a.xy[c] >> 16)) | a.zt[c]) & FIX_FINE;
+    all = all && (up & 0xffffu) && (up >> 16) && (low & 0xffffu) && (low >> 16);
+  }
+  return all || a.any == 0;
+}
+
+// T 2^(E - 1023 - 58) as a double, rounded to nearest
 __host__ __device__ __forceinline__ double fix_double(long long t, int E) {
   const long long s = t >> 63;
   const unsigned long long m = (unsigned long long)((t ^ s) - s);
@@ -334,7 +429,7 @@ __host__ __device__ __forceinline__ double fix_double(long long t, int E) {
   const int lz = m ? __builtin_clzll(m) : 64;
 #endif
   const unsigned long long n = m << (lz & 63);
-  unsigned long long b = ((unsigned long long)(E + 7 - lz) << 52) + (n >> 11) + ((n >> 10) & 1);
+  unsigned long long b = ((unsigned long long)(E + 4 - lz) << 52) + (n >> 11) + ((n >> 10) & 1);
   b |= (unsigned long long)s & 0x8000000000000000ull;
   if (m == 0) b = 0;
   double d;

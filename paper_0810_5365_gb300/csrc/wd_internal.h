@@ -17,7 +17,7 @@ namespace wd {
 // Register budgets from sweeps on GB300 (32^3x64): FP32 is fastest with 7
 // resident 128-thread blocks per SM (<= 72 registers), FP16 with 6 (<= 80
 // registers, two hops of loads in flight; 5 and 7 are slower); the FP64
-// fixed-point hops get 3 (168 registers; 24^3x48: 175 us, 2 blocks 209, 4
+// fixed-point hops get 3 (168 registers; 24^3x48, first form: 175 us, 2 blocks 209, 4
 // blocks spill and take 185).
 #ifndef WD_DSLASH_MINB_F64
 #define WD_DSLASH_MINB_F64 3
