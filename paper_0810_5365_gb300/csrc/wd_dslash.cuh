@@ -579,13 +579,13 @@ __device__ __forceinline__ void hop_fix(FixSite& fx, int mu, const void* __restr
     case 2: project<2, S>(psi, h); break;
     default: project<3, S>(psi, h); break;
   }
-  fix_hop<S, FWD, RC>(fx, mu, h, u, flip, unit);
+  fix_hop<S, FWD, RC, RC == 18>(fx, mu, h, u, flip, unit);
 }
 
 // The eight hops of one FP64 site: fixed point, or the FP64 chain where the
 // values do not fit it.  24^3x48, one parity, us per launch: FP64 chain 537
 // (recon 18) and 686 (recon 12, which rebuilds row 2 on the FP64 pipe), fixed
-// point 185 and 212.  What bounds it now: the integer pipes (ALU 42 % busy)
+// point 187 and 212.  What bounds it now: the integer pipes (ALU 42 % busy)
 // through the latency of dependent instructions, with 12 warps per SM at 168
 // registers; 8 or 16 warps (255 registers, or 128 and spills) are slower.  The
 // directions are a loop, not unrolled: eight copies of the hop (200 KB of

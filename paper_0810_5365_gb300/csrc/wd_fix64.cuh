@@ -11,7 +11,7 @@
 // Formats (E: the site's scale, a biased exponent, e = E - 1023; no projected
 // component seen so far is 1.5 2^e or more):
 //   half spinor  h = H 2^(e-61), |H| < 1.5 2^61
-//   link         u = V 2^-61,    |V| < 2^61 (1 + 2^-20)
+//   link         u = V 2^(el-61), |V| < 2^61 (1 + 2^-20), el 0 for SU(3) (fix_hop)
 //   products     t = T 2^(e-58), below 2^60 each (fix_ok; rows of a norm of up
 //                to one cannot give more), so that the sum of eight fits 64 bits
 // H and V are cut into two signed 32-bit limbs, x = x.h 2^32 + x.l, and
@@ -32,11 +32,11 @@
 // error is 0.41 of the chain's for products of one size and 0.95 of it at that
 // line (tests/host/fix64_small_check.cu; 2^-6 would be 1.5 times the chain's).
 //
-// A site also falls back to the FP64 chain when a value does not fit: |u| above
-// 1 or a link that is small throughout (not SU(3)), infinities, NaN, or
-// exponents near the ends of the range.  Where that happens the site costs both
-// (24^3x48, us, all sites in the chain / none: 660 / 185 with 18-real links,
-// 813 / 212 with 12).  On Gaussian fields and on solutions and residuals of
+// A site also falls back to the FP64 chain when a value does not fit: 12-real
+// links with |u| above 1 or small throughout (not SU(3)), 18-real ones beyond
+// 2^64, infinities, NaN, or exponents near the ends of the range.  Where that
+// happens the site costs both (24^3x48, us, all sites in the chain / none: 660
+// / 187 with 18-real links, 812 / 212 with 12).  On Gaussian fields and on solutions and residuals of
 // Gaussian sources no site does; on the propagator of a point source 0.1 to 2 %
 // of the warps hold one with links of mean 0.94 (216 to 230 us, 18-real), most
 // of them with smoother links (exp(0.15 i H): 410 to 560).
@@ -45,7 +45,8 @@
 // 32-bit words: on a 64-bit variable the compiler took 16), 216 multiply-adds,
 // about 150 for the sums and their sizes and 60 for the scale.  The sizes and
 // the three bits that T has for the line at 2^-5 (a carry between the halves of
-// a row) cost 6 to 9 %: 174 -> 185 us and, with 12-real links, 193 -> 212; at
+// a row) cost 6 to 9 %: 174 -> 185 us and, with 12-real links, 193 -> 212 (the
+// links' own scale another 2 us with 18-real ones); at
 // 2^-3 without those bits the propagators above took the chain everywhere.
 #pragma once
 
@@ -83,6 +84,7 @@ constexpr unsigned FIX_FULL = 0xe000e000u;
 constexpr unsigned FIX_ROOM = 0x80000u;
 constexpr unsigned FIX_UMAX = 0x3ff00000u;  // high words of |u| < 1 + 2^-20 ...
 constexpr unsigned FIX_UMIN = 0x3fc00000u;  // ... and of 1/8 (an SU(3) row has a real >= 0.23)
+constexpr int FIX_LINK = 64;  // largest |el| of a link; zero and tiny links count as 2^-64
 
 __host__ __device__ __forceinline__ unsigned long long d_bits(double x) {
   unsigned long long b;
@@ -193,7 +195,9 @@ __host__ __device__ __forceinline__ unsigned fix_sizes(const FixSite& a) {
 // through the products like any other: they come out as zero, a link that does
 // not fit is seen (0 times NaN is NaN), and the time of a launch, which the
 // tuners compare, does not depend on how much of a field is zero.
-__host__ __device__ __forceinline__ void fix_scale(FixSite& acc, const cx<double> (&h)[6]) {
+// el: the link's exponent (fix_hop).
+__host__ __device__ __forceinline__ void fix_scale(FixSite& acc, const cx<double> (&h)[6],
+                                                   int el) {
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k < 6; k++) {
@@ -210,7 +214,7 @@ __host__ __device__ __forceinline__ void fix_scale(FixSite& acc, const cx<double
     for (int k = 0; k < 6; k++) lows |= d_bits(h[k].r) | d_bits(h[k].i);
     acc.bad |= (unsigned)lows;
   }
-  const int e = (int)((m + FIX_ROOM) >> 20);
+  const int e = (int)((m + FIX_ROOM) >> 20) + el;
   if (e > acc.E) {
     const int d = e - acc.E < 63 ? e - acc.E : 63;
     acc.E = e;
@@ -322,15 +326,34 @@ __host__ __device__ __forceinline__ void fix_expand(FixSite& acc, int mu, int c,
 // times the link u (RC reals as stored; not read when unit), added to the
 // site's sums.  Colour by colour, so that only one row of products is live
 // beside the sums.
-template <int S, bool FWD, int RC>
+//
+// SIZED (18-real links): a link that is not of order one (tadpole-scaled or
+// smeared ones, anisotropic actions) is held as 2^el times one that is, and its
+// products scale the site: without it each site next to such a link took the
+// chain after its fixed-point pass, 24^3x48 651 us a launch where the chain
+// alone took 537, and now 188.  12-real links are SU(3), others take the chain: row 2, a
+// product of the rows, does not scale with them.
+template <int S, bool FWD, int RC, bool SIZED = false>
 __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<double> (&h)[6],
                                                  const double (&u)[RC], bool flip, bool unit) {
-  fix_scale(acc, h);
+  static_assert(!SIZED || RC == 18, "12-real links have no scale of their own");
+  unsigned um = 0;
+  int el = 0;
+  if (SIZED && !unit) {
+#pragma unroll
+    for (int k = 0; k < RC; k++) fix_link_max(um, d_bits(u[k]));
+    if (um > FIX_UMAX || um < FIX_UMIN) {
+      el = (int)((um + 0xfffffu) >> 20) - 1023;
+      acc.bad |= el > FIX_LINK ? 1u : 0u;
+      el = el > FIX_LINK ? FIX_LINK : el < -FIX_LINK ? -FIX_LINK : el;
+    }
+  }
+  fix_scale(acc, h, el);
   Limb H[6][2];
 #pragma unroll
   for (int k = 0; k < 6; k++) {
-    H[k][0] = fix_limbs(d_bits(h[k].r), acc.E + 2);
-    H[k][1] = fix_limbs(d_bits(h[k].i), acc.E + 2);
+    H[k][0] = fix_limbs(d_bits(h[k].r), acc.E - el + 2);
+    H[k][1] = fix_limbs(d_bits(h[k].i), acc.E - el + 2);
   }
   if (flip) {
 #pragma unroll
@@ -348,7 +371,6 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
     return;
   }
   Limb U[9][2];
-  unsigned um = 0;
   if (RC == 12) {
 #pragma unroll
     for (int k = 0; k < RC; k++) {
@@ -382,8 +404,8 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
         if (RC == 12) {
           v[d][j] = U[k][j];
         } else {
-          fix_link_max(um, d_bits(u[2 * k + j]));
-          v[d][j] = fix_limbs(d_bits(u[2 * k + j]), 1023 + 2);
+          if (!SIZED) fix_link_max(um, d_bits(u[2 * k + j]));
+          v[d][j] = fix_limbs(d_bits(u[2 * k + j]), 1023 + el + 2);
         }
       }
     }
@@ -392,7 +414,7 @@ __host__ __device__ __forceinline__ void fix_hop(FixSite& acc, int mu, const cx<
     fix_row<FWD>(r1, i1, v, &H[3]);
     fix_expand<S>(acc, mu, c, r0, i0, r1, i1);
   }
-  acc.bad |= (um > FIX_UMAX || um < FIX_UMIN) ? 1u : 0u;
+  if (!SIZED) acc.bad |= (um > FIX_UMAX || um < FIX_UMIN) ? 1u : 0u;
 }
 
 // whether the site's sums are valid (else: the FP64 chain)
