@@ -910,8 +910,9 @@ struct Alloc {
   }
 };
 
-// Scratch of the synchronous network calls (wd_nn_apply*, wd_nn_wgrad): kept
-// between calls, since a cudaMalloc/cudaFree pair of its size costs as much as
+// Scratch of the synchronous network calls (wd_nn_apply*, wd_nn_layer,
+// wd_nn_wgrad), the error flag of their bounded waits included: kept between
+// calls, since a cudaMalloc/cudaFree pair of its size costs as much as
 // the kernels (wd_nn_apply_ex on 32^3x64, BF16: 0.9 ms of kernels, 1.0 ms of
 // allocation).  One call at a time has it: a call that finds it taken by
 // another host thread allocates its own.  Every call returns it with its
@@ -924,7 +925,8 @@ struct NnScratch {
   char* at = nullptr;
   bool idle = false;  // the call has synchronised its stream
   bool held = false;  // the call has the kept scratch
-  cudaStream_t st = state().stream;
+  const cudaStream_t st;
+  explicit NnScratch(cudaStream_t stream) : st(stream) {}
   Alloc own;          // a request above NN_SCRATCH_KEEP, or the kept one taken
   ~NnScratch() {
     if (!idle) cudaStreamSynchronize(st);
@@ -951,6 +953,13 @@ struct NnScratch {
     }
     at = (char*)s.nn_scratch;
     return cudaSuccess;
+  }
+  // get, and this call's own error flag at its start, cleared
+  cudaError_t get_with_flag(size_t bytes, int** flag) {
+    const cudaError_t e = get(256 + bytes);
+    if (e != cudaSuccess) return e;
+    *flag = (int*)take(256);
+    return cudaMemsetAsync(*flag, 0, sizeof(int), st);
   }
   // the next part (256-byte multiples)
   void* take(size_t bytes) {
@@ -1018,14 +1027,13 @@ cudaError_t full_op(int prec, int recon, const void* gauge, void* out, const voi
 int nn_apply_impl(void* out, const void* in, const float* w, const void* gauge, const int dims[4]) {
   const Geom g = make_geom(dims);
   cudaStream_t st = state().stream;
-  NnScratch sc;
+  NnScratch sc(st);
   NnBuffers B;
   B.bytes8 = 2 * nn_half_bytes(g.Vh_pad, 8);
-  NCK(sc.get(2 * B.bytes8));
+  int* flag = nullptr;
+  NCK(sc.get_with_flag(2 * B.bytes8, &flag));
   B.h1 = sc.take(B.bytes8);
   B.h2 = sc.take(B.bytes8);
-  int* flag = nullptr;
-  NCK(device_flag(&flag, st));
   NCK(nn_forward(g, gauge, w, in, out, B, flag, st));
   int hflag = 0;
   NCK(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1042,15 +1050,14 @@ int nn_apply_ex_impl(void* out, const void* in, const float* w, const void* gaug
   const Geom g = make_geom(dims);
   cudaStream_t st = state().stream;
   const bool even = (flags & 2) != 0, bf16 = (flags & 1) != 0;
-  NnScratch sc;
+  NnScratch sc(st);
   NnBuffers B;
   B.bytes8 = 2 * (bf16 ? nn_half_bytes_bf16(g.Vh_pad, 8) : nn_half_bytes(g.Vh_pad, 8));
   const size_t gbytes = bf16 ? nn_gauge_bytes_bf16(g.Vh_pad) : 0;
-  NCK(sc.get(2 * B.bytes8 + round_up(gbytes, 256)));
+  int* flag = nullptr;
+  NCK(sc.get_with_flag(2 * B.bytes8 + round_up(gbytes, 256), &flag));
   B.h1 = sc.take(B.bytes8);
   B.h2 = sc.take(B.bytes8);
-  int* flag = nullptr;
-  NCK(device_flag(&flag, st));
   if (bf16) {
     void* gbf = sc.take(gbytes);
     NCK(nn_gauge_bf16(gbf, gauge, g, st));
@@ -1071,12 +1078,14 @@ int nn_layer_impl(void* out, const void* in, const float* w, int cin, int cout, 
                   const int dims[4]) {
   const Geom g = make_geom(dims);
   cudaStream_t st = state().stream;
+  NnScratch sc(st);
   int* flag = nullptr;
-  NCK(device_flag(&flag, st));
+  NCK(sc.get_with_flag(0, &flag));
   NCK(nn_layer(cin, cout, g, gauge, in, out, w, flag, st));
   int hflag = 0;
   NCK(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   NCK(cudaStreamSynchronize(st));
+  sc.idle = true;
   return hflag ? WD_ERR_TIMEOUT : WD_OK;
 }
 
@@ -1084,13 +1093,12 @@ int nn_wgrad_impl(float* grad, const void* in, const void* delta, int cin, int c
                   const void* gauge, const int dims[4]) {
   const Geom g = make_geom(dims);
   cudaStream_t st = state().stream;
-  NnScratch sc;
+  NnScratch sc(st);
   const int ntile = 2 * ((g.Vh + NN_TILE - 1) / NN_TILE);
   const size_t pbytes = (size_t)ntile * NN_NDIR * cout * cin * 2 * sizeof(float);
-  NCK(sc.get(round_up(pbytes, 256)));
-  void* part = sc.take(pbytes);
   int* flag = nullptr;
-  NCK(device_flag(&flag, st));
+  NCK(sc.get_with_flag(round_up(pbytes, 256), &flag));
+  void* part = sc.take(pbytes);
   NCK(nn_wgrad(cin, cout, g, gauge, in, delta, (float*)part, grad, 0, flag, st));
   int hflag = 0;
   NCK(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
