@@ -117,8 +117,8 @@ const char *wd_error_string(int status);
 int wd_last_cuda_error(void);
 
 /* Free the library's cached workspace (solver fields, reduction scratch, the
- * network calls' scratch of at most 1 GiB, captured graphs).  Caller buffers
- * are untouched.  Safe to call twice. */
+ * network calls' scratch of at most 1 GiB unless another host thread's call has
+ * it, captured graphs).  Caller buffers are untouched.  Safe to call twice. */
 void wd_finalize(void);
 
 /* ------------------------------------------------------------------ */

@@ -128,13 +128,11 @@ void wd_finalize(void) {
   if (s.partials) cudaFree(s.partials);
   if (s.counter) cudaFree(s.counter);
   if (s.dev_flag) cudaFree(s.dev_flag);
-  if (s.nn_scratch) cudaFree(s.nn_scratch);
-  s.nn_scratch = nullptr;
-  s.nn_scratch_bytes = 0;
   s.partials = nullptr;
   s.counter = nullptr;
   s.dev_flag = nullptr;
   s.partials_cap = 0;
+  drop_nn_scratch();
 }
 
 size_t wd_spinor_bytes(const int dims[4], int parity, int prec) {

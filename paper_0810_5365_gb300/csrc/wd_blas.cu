@@ -71,6 +71,17 @@ cudaError_t ensure_scratch(size_t doubles) {
   return cudaSuccess;
 }
 
+bool drop_nn_scratch() {
+  State& s = state();
+  if (s.nn_scratch_taken.exchange(true)) return false;
+  const bool had = s.nn_scratch != nullptr;
+  if (had) cudaFree(s.nn_scratch);
+  s.nn_scratch = nullptr;
+  s.nn_scratch_bytes = 0;
+  s.nn_scratch_taken.store(false);
+  return had;
+}
+
 cudaError_t device_flag(int** flag, cudaStream_t st) {
   State& s = state();
   if (!s.dev_flag) {

@@ -219,6 +219,10 @@ cudaError_t axpby(double a, const void* x, double b, void* y, const Geom& g, int
 // zeroed device flag for bounded device-side waits (allocated on first use)
 cudaError_t device_flag(int** flag, cudaStream_t st);
 
+// free the network calls' kept scratch; false when there is none or a call has
+// it (of another host thread: it stays then)
+bool drop_nn_scratch();
+
 // tensor-core GEMM (wd_tcgemm.cu)
 cudaError_t tc_gemm_bf16(const void* A, const void* B, float* D, int M, int K, int N, int* err,
                          cudaStream_t st);
