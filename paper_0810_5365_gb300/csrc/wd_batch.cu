@@ -176,7 +176,7 @@ cudaError_t mrhs_lanes(int prec, const MrhsBatch& bt, int recon, bool dagger, co
   size_t total = 256 + (size_t)MRHS_MAX_PROBLEMS * MRHS_MAX * sizeof(double);
   for (int j = 0; j < bt.nprob; j++) total += ((size_t)bt.p[j].nrhs * bt.p[j].s_out + 255) / 256 * 256;
   char* buf = nullptr;
-  if (cudaMalloc(&buf, total) != cudaSuccess) {
+  if (device_malloc(&buf, total) != cudaSuccess) {
     cudaGetLastError();  // no room to tune: keep the default shape
     return cudaSuccess;
   }
@@ -839,7 +839,7 @@ void free_ctx(BatchCtx& c) {
 }
 
 cudaError_t dalloc(BatchCtx& c, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = device_malloc(p, bytes);
   if (e == cudaSuccess) c.allocs.push_back(*p);
   return e;
 }

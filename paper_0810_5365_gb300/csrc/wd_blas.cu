@@ -52,7 +52,7 @@ int blas_grid(long long n, int bs) {
 cudaError_t ensure_scratch(size_t doubles) {
   State& s = state();
   if (!s.counter) {
-    cudaError_t e = cudaMalloc(&s.counter, 256);
+    cudaError_t e = device_malloc(&s.counter, 256);
     if (e != cudaSuccess) return e;
     e = cudaMemset(s.counter, 0, 256);
     if (e != cudaSuccess) return e;
@@ -65,7 +65,7 @@ cudaError_t ensure_scratch(size_t doubles) {
     s.partials = nullptr;
     s.partials_cap = 0;
   }
-  cudaError_t e = cudaMalloc(&s.partials, cap * sizeof(double));
+  cudaError_t e = device_malloc(&s.partials, cap * sizeof(double));
   if (e != cudaSuccess) return e;
   s.partials_cap = cap;
   return cudaSuccess;
@@ -82,10 +82,17 @@ bool drop_nn_scratch() {
   return had;
 }
 
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_nn_scratch()) e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();  // (returned here: not to the next launch's check)
+  return e;
+}
+
 cudaError_t device_flag(int** flag, cudaStream_t st) {
   State& s = state();
   if (!s.dev_flag) {
-    cudaError_t e = cudaMalloc(&s.dev_flag, 256);
+    cudaError_t e = device_malloc(&s.dev_flag, 256);
     if (e != cudaSuccess) return e;
   }
   *flag = s.dev_flag;

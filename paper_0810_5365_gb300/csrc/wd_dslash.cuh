@@ -929,7 +929,7 @@ cudaError_t dslash_block(const DslashArgs& a, int recon, bool dagger, cudaStream
   if (e != cudaSuccess) return e;
   if (cs != cudaStreamCaptureStatusNone) return cudaSuccess;
   void* tmp = nullptr;
-  if (cudaMalloc(&tmp, spinor_half_bytes(a.g, P)) != cudaSuccess) {
+  if (device_malloc(&tmp, spinor_half_bytes(a.g, P)) != cudaSuccess) {
     cudaGetLastError();  // no room to tune: keep the default
     return cudaSuccess;
   }

@@ -223,6 +223,14 @@ cudaError_t device_flag(int** flag, cudaStream_t st);
 // it (of another host thread: it stays then)
 bool drop_nn_scratch();
 
+// cudaMalloc; where the device's memory does not suffice, again without the
+// kept scratch (keeping it takes no allocation from a call that had room before)
+cudaError_t device_malloc(void** p, size_t bytes);
+template <typename T>
+cudaError_t device_malloc(T** p, size_t bytes) {
+  return device_malloc((void**)p, bytes);
+}
+
 // tensor-core GEMM (wd_tcgemm.cu)
 cudaError_t tc_gemm_bf16(const void* A, const void* B, float* D, int M, int K, int N, int* err,
                          cudaStream_t st);

@@ -901,7 +901,7 @@ namespace {
 struct Alloc {
   std::vector<void*> ptrs;
   cudaError_t get(void** p, size_t bytes) {
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = device_malloc(p, bytes);
     if (e == cudaSuccess) ptrs.push_back(*p);
     return e;
   }
@@ -944,7 +944,7 @@ struct NnScratch {
       if (s.nn_scratch) cudaFree(s.nn_scratch);
       s.nn_scratch = nullptr;
       s.nn_scratch_bytes = 0;
-      if ((e = cudaMalloc(&s.nn_scratch, bytes)) != cudaSuccess) {
+      if ((e = device_malloc(&s.nn_scratch, bytes)) != cudaSuccess) {
         s.nn_scratch = nullptr;
         return e;
       }

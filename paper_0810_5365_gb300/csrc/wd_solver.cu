@@ -505,26 +505,26 @@ static int ws_ensure(const int dims[4], int sprec, int srecon, int orecon) {
   w.g = g;
   size_t h64 = spinor_half_bytes(g, WD_F64), hs = spinor_half_bytes(g, sprec);
   size_t hx = spinor_half_bytes(g, sloppy_x_prec(sprec));
-  WD_CK(cudaMalloc(&w.g64, gauge_bytes(g, WD_F64, orecon)));
+  WD_CK(device_malloc(&w.g64, gauge_bytes(g, WD_F64, orecon)));
   if (sprec == WD_F64 && srecon == orecon)
     w.gs = w.g64;
   else
-    WD_CK(cudaMalloc(&w.gs, gauge_bytes(g, sprec, srecon)));
-  WD_CK(cudaMalloc(&w.b64, 2 * h64));
-  WD_CK(cudaMalloc(&w.x64, 2 * h64));
-  WD_CK(cudaMalloc(&w.rf64, 2 * h64));
-  WD_CK(cudaMalloc(&w.bhat, h64));
-  WD_CK(cudaMalloc(&w.r64, h64));
-  WD_CK(cudaMalloc(&w.t64, h64));
-  WD_CK(cudaMalloc(&w.p, hs));
-  WD_CK(cudaMalloc(&w.q, hs));
-  WD_CK(cudaMalloc(&w.r, hs));
-  WD_CK(cudaMalloc(&w.s, hs));
-  WD_CK(cudaMalloc(&w.ts, hs));
-  WD_CK(cudaMalloc(&w.t, hs));
-  WD_CK(cudaMalloc(&w.r0, hs));
-  WD_CK(cudaMalloc(&w.xs, hx));
-  WD_CK(cudaMalloc(&w.sc, sizeof(CgScalars)));
+    WD_CK(device_malloc(&w.gs, gauge_bytes(g, sprec, srecon)));
+  WD_CK(device_malloc(&w.b64, 2 * h64));
+  WD_CK(device_malloc(&w.x64, 2 * h64));
+  WD_CK(device_malloc(&w.rf64, 2 * h64));
+  WD_CK(device_malloc(&w.bhat, h64));
+  WD_CK(device_malloc(&w.r64, h64));
+  WD_CK(device_malloc(&w.t64, h64));
+  WD_CK(device_malloc(&w.p, hs));
+  WD_CK(device_malloc(&w.q, hs));
+  WD_CK(device_malloc(&w.r, hs));
+  WD_CK(device_malloc(&w.s, hs));
+  WD_CK(device_malloc(&w.ts, hs));
+  WD_CK(device_malloc(&w.t, hs));
+  WD_CK(device_malloc(&w.r0, hs));
+  WD_CK(device_malloc(&w.xs, hx));
+  WD_CK(device_malloc(&w.sc, sizeof(CgScalars)));
   WD_CK(cudaMemset(w.sc, 0, sizeof(CgScalars)));
   WD_CK(cudaMallocHost(&w.sc_host, sizeof(CgScalars)));
   WD_CK(cudaStreamCreateWithFlags(&w.cap, cudaStreamNonBlocking));
@@ -779,22 +779,22 @@ int solve_impl(double* x, const double* b, const double* gauge, double kappa, co
   // ---- stage and pack the inputs ----
   const double* bdev = b;
   if (!is_device_ptr(b)) {
-    if (!w.canon_spinor) WD_CK(cudaMalloc(&w.canon_spinor, V * 24 * sizeof(double)));
+    if (!w.canon_spinor) WD_CK(device_malloc(&w.canon_spinor, V * 24 * sizeof(double)));
     WD_CK(cudaMemcpyAsync(w.canon_spinor, b, V * 24 * sizeof(double), cudaMemcpyHostToDevice, st));
     bdev = w.canon_spinor;
   }
   const double* gdev = gauge;
   if (!is_device_ptr(gauge)) {
-    if (!w.canon_gauge) WD_CK(cudaMalloc(&w.canon_gauge, 4 * V * 18 * sizeof(double)));
+    if (!w.canon_gauge) WD_CK(device_malloc(&w.canon_gauge, 4 * V * 18 * sizeof(double)));
     WD_CK(cudaMemcpyAsync(w.canon_gauge, gauge, 4 * V * 18 * sizeof(double),
                           cudaMemcpyHostToDevice, st));
     gdev = w.canon_gauge;
   }
   if (P.gauge_fix) {
     // solve D[U'] x' = omega b in temporal gauge, then x = omega^+ x'
-    if (!w.gf_gauge) WD_CK(cudaMalloc(&w.gf_gauge, 4 * V * 18 * sizeof(double)));
-    if (!w.gf_omega) WD_CK(cudaMalloc(&w.gf_omega, V * 18 * sizeof(double)));
-    if (!w.gf_spinor) WD_CK(cudaMalloc(&w.gf_spinor, V * 24 * sizeof(double)));
+    if (!w.gf_gauge) WD_CK(device_malloc(&w.gf_gauge, 4 * V * 18 * sizeof(double)));
+    if (!w.gf_omega) WD_CK(device_malloc(&w.gf_omega, V * 18 * sizeof(double)));
+    if (!w.gf_spinor) WD_CK(device_malloc(&w.gf_spinor, V * 24 * sizeof(double)));
     WD_CK(gauge_fix_temporal(w.gf_gauge, w.gf_omega, gdev, g, st));
     WD_CK(rotate_spinor(w.gf_spinor, bdev, w.gf_omega, g, 0, st));
     gdev = w.gf_gauge;
@@ -809,7 +809,7 @@ int solve_impl(double* x, const double* b, const double* gauge, double kappa, co
   if (P.use_initial_guess) {
     const double* xdev = x;
     if (!x_dev) {
-      if (!w.canon_spinor) WD_CK(cudaMalloc(&w.canon_spinor, V * 24 * sizeof(double)));
+      if (!w.canon_spinor) WD_CK(device_malloc(&w.canon_spinor, V * 24 * sizeof(double)));
       WD_CK(cudaMemcpyAsync(w.canon_spinor, x, V * 24 * sizeof(double), cudaMemcpyHostToDevice, st));
       xdev = w.canon_spinor;
     }
@@ -971,7 +971,7 @@ int solve_impl(double* x, const double* b, const double* gauge, double kappa, co
             &w.sc->res_o, st));
   // ---- unpack the solution ----
   double* xdev = x_dev ? x : w.canon_spinor;
-  if (!x_dev && !w.canon_spinor) WD_CK(cudaMalloc(&w.canon_spinor, V * 24 * sizeof(double)));
+  if (!x_dev && !w.canon_spinor) WD_CK(device_malloc(&w.canon_spinor, V * 24 * sizeof(double)));
   xdev = x_dev ? x : w.canon_spinor;
   WD_CK(unpack_spinor(xdev, w.x64, g, WD_FULL, WD_F64, st));
   if (P.gauge_fix) WD_CK(rotate_spinor(xdev, xdev, w.gf_omega, g, 1, st));
