@@ -8,7 +8,10 @@ output parity each step.  Effective Gflops use the nominal 1320 flops per
 site (reconstruction work not counted, as the paper counts its effective
 Gflops, section "Performance").
 
-The JSON line (rank 0) carries, besides metric/value/unit:
+The JSON line (rank 0) is short (headline_line: under 3000 characters, so that
+whoever keeps only the end of a log keeps it whole).  The sections that it
+names only in its summary go, in full, to the file given by --detail.
+Measured are, besides metric/value/unit:
   roofline      achieved GB/s against the measured copy peak (and the nominal
                 8 TB/s), with the DRAM traffic per launch from the committed
                 ncu counters while the kernel sources are unchanged;
@@ -19,7 +22,7 @@ The JSON line (rank 0) carries, besides metric/value/unit:
   e2e           the headline through the C ABI with pinned host buffers and
                 the copies inside the timed region (pipelined over streams);
   clocks        SM clocks and throttle reasons sampled during the timing;
-  summary       the figures of the sections below in a few short keys;
+  summary       the figures of the sections in a few short keys;
   cpu_baseline  the FP64 oracle on the host cores (and one thread), plus the
                 oracle's plain FP64 CG to 1e-10 on 24^3x48, timed whole;
   solve         time to a 1e-10 true residual on 24^3x48: mixed-precision CG
@@ -238,11 +241,33 @@ def oracle_cg_full(maxiter=4000):
             "problem": "24^3x48, kappa 0.137, complex Gaussian b (seed 2025), tol 1e-10"}
 
 
+def short(v):
+    """Numbers to five digits, through dicts and lists."""
+    if isinstance(v, dict):
+        return {k: short(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [short(x) for x in v]
+    return float(f"{v:.5g}") if isinstance(v, float) else v
+
+
+def headline_line(line):
+    """The JSON line that is printed: the headline with its own checks in full,
+    of the other sections the summary."""
+    keep = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+            "scaling", "vs_baseline", "dtype", "data", "config", "dslash_gbs", "gpu_launches", "clocks")
+    out = {k: line[k] for k in keep}
+    drop = {"roofline": ("frac_of_nominal_8tbs",), "e2e": ("overlap",), "mhat": ("note", "unit", "steps"),
+            "graph": ("note", "unit"), "cpu_baseline": ("sample", "oracle_cg_24x24x24x48")}
+    for k, without in drop.items():
+        if k in line:
+            out[k] = {a: b if k == "e2e" else short(b) for a, b in line[k].items() if a not in without}
+    out["summary"] = compact_summary(line)
+    return out
+
+
 def compact_summary(line):
-    """The figures of the sub-sections in a few short keys, so that they sit
-    near the start of the JSON line."""
-    sm = {"dslash_f32_frac": round(line["roofline"]["frac"], 3),
-          "variants_frac": {k: round(v["frac"], 3) for k, v in line["variants"].items()},
+    """The figures of the sub-sections in a few short keys."""
+    sm = {"variants_frac": {k: round(v["frac"], 3) for k, v in line["variants"].items()},
           "variants_us": {k: round(v["ms_per_step"] * 1e3, 1) for k, v in line["variants"].items()}}
     if "solve" in line:
         sm["solve_24x48_s_iters_speedup"] = {
@@ -1026,8 +1051,7 @@ def run_ours(args, rank, world, local):
         if name == "f16_staged":
             line["variants"][name]["note"] = (
                 "FP16 with the +-z and +-t neighbour spinors staged in shared memory by "
-                "bulk asynchronous (TMA) copies, one mbarrier per warp; bit-identical to f16, "
-                "and the kernel the CTA-size tuner chooses for plain FP16 calls on this lattice")
+                "bulk asynchronous (TMA) copies, one mbarrier per warp; bit-identical to f16")
         line["gpu_launches"] += st
     line["e2e"] = {"value": FLOPS_PER_SITE * Vh * k_e2e * world / dt_e2e / 1e9, "unit": "Gflops",
                    "steps": k_e2e, "h2d_bytes_per_step": nb, "d2h_bytes_per_step": nb,
@@ -1054,14 +1078,10 @@ def run_ours(args, rank, world, local):
             oc["gpu_mixed_f16_speedup"] = oc["wall_s"] / oc["gpu_mixed_f16_cg_s"]
             line["cpu_baseline"]["oracle_cg_24x24x24x48"] = oc
     if rank == 0:
-        # the compact summary right after the config, ahead of the long sections
-        head = {}
-        for k, v in line.items():
-            head[k] = v
-            if k == "config":
-                head["summary"] = compact_summary(line)
-        line = head
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f, indent=1)
+        print(json.dumps(headline_line(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
@@ -1078,6 +1098,7 @@ def main():
     ap.add_argument("--no-solve", action="store_true", help="skip the 24^3x48 solver comparison")
     ap.add_argument("--no-oracle-cg", action="store_true",
                     help="skip the oracle's full FP64 CG timing (about 100 s of host time)")
+    ap.add_argument("--detail", metavar="FILE", help="write every section in full to FILE")
     ap.add_argument("--profile", choices=["mrhs", "solve_f32", "solve_f16", "batch",
                                           "batch_persistent", "fcg", "train", "nn", "nn_bf16",
                                           "staged"],
