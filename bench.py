@@ -740,6 +740,8 @@ def profile_case(name):
                   tensor-core weight-gradient kernels);
     ``nn``        2 applications of the series-initialised network (three
                   tensor-core layers) on 16^3x32;
+    ``f64``       4 FP64 parity dslashes on 24^3x48 with 12-real links, then 4
+                  with 18-real ones (128-site CTAs forced, so no tuning runs);
     ``staged``    4 FP16 parity dslashes on 32^3x64 with the far neighbours
                   staged by bulk copies (WD_STAGE_NEIGHBOURS), then 4 with the
                   unstaged kernel (128-site CTAs forced, so no tuning runs)."""
@@ -778,6 +780,21 @@ def profile_case(name):
             for _ in range(4):
                 W.wd_dslash_ex(a[:h], a[h:], g, W.WD_EVEN, 0, -KAPPA, None, 0.0, None, 0.0,
                                None, dims, W.WD_F16, recon)
+        W.wd_dslash_set_block(0)
+    elif name == "f64":
+        dims = SOLVE_DIMS
+        Ud = torch.from_numpy(fields.su3_links(dims).view(np.float64).reshape(-1)).cuda()
+        src = torch.from_numpy(fields.gaussian_spinor(dims).view(np.float64).reshape(-1)).cuda()
+        a = W.alloc_spinor(dims, W.WD_FULL, W.WD_F64)
+        W.wd_pack_spinor(a, src, dims, W.WD_FULL, W.WD_F64)
+        h = W.wd_spinor_bytes(dims, W.WD_EVEN, W.WD_F64)
+        W.wd_dslash_set_block(128)
+        for recon in (12, 18):
+            g = W.alloc_gauge(dims, W.WD_F64, recon)
+            W.wd_pack_gauge(g, Ud, dims, W.WD_F64, recon)
+            for _ in range(4):
+                W.wd_dslash_ex(a[:h], a[h:], g, W.WD_EVEN, 0, -KAPPA, None, 0.0, None, 0.0,
+                               None, dims, W.WD_F64, recon)
         W.wd_dslash_set_block(0)
     elif name in ("solve_f32", "solve_f16"):
         dims = SOLVE_DIMS
@@ -1101,7 +1118,7 @@ def main():
     ap.add_argument("--detail", metavar="FILE", help="write every section in full to FILE")
     ap.add_argument("--profile", choices=["mrhs", "solve_f32", "solve_f16", "batch",
                                           "batch_persistent", "fcg", "train", "nn", "nn_bf16",
-                                          "staged"],
+                                          "staged", "f64"],
                     help="run a short fixed workload for an ncu capture and exit")
     args = ap.parse_args()
     if args.profile:

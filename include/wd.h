@@ -163,6 +163,10 @@ int wd_convert_spinor(void *dst, int dst_prec, const void *src, int src_prec,
  *     out = in - kappa * H in = D in    (packed full fields).
  * gauge is packed with the same prec and recon 12 (use wd_dslash_ex for
  * recon 18).  out must not alias in (WD_ERR_ALIAS).
+ * WD_F64 sums the hops of a site in 64-bit fixed point where that gives each
+ * component at least the bits of FP64 arithmetic, else in FP64 (infinities and
+ * NaN, components far below the site's largest neighbour, 12-real links that are
+ * not SU(3)); such sites take about 3.5 times as long.
  */
 int wd_dslash(void *out, const void *in, const void *gauge, double kappa,
               int parity, const int dims[4], int prec);
@@ -289,7 +293,8 @@ int wd_dslash_set_block(int sites);
  * wd_dslash_ex, wd_mhat, wd_dslash_mrhs, wd_norm2, wd_cdot and wd_axpby, and
  * those of the solvers' iterations where it pays (not in the captured
  * iterations of medium lattices, of FP64 and of wd_solve_batch, nor for FP64
- * axpby), are programmatic dependent launches.  The kernel first waits until
+ * axpby, nor for the FP64 norm of a field that does not fill the GPU), are
+ * programmatic dependent launches.  The kernel first waits until
  * the previous kernel of the stream has completed and its writes are visible,
  * before it reads or writes any memory, then lets the next kernel be scheduled
  * once all of its own CTAs have got that far.  So consecutive launches

@@ -34,20 +34,22 @@
 //
 // A site also falls back to the FP64 chain when a value does not fit: 12-real
 // links with |u| above 1 or small throughout (not SU(3)), 18-real ones beyond
-// 2^64, infinities, NaN, or exponents near the ends of the range.  Where that
-// happens the site costs both (24^3x48, us, all sites in the chain / none: 660
-// / 187 with 18-real links, 812 / 212 with 12).  On Gaussian fields and on solutions and residuals of
-// Gaussian sources no site does; on the propagator of a point source 0.1 to 2 %
-// of the warps hold one with links of mean 0.94 (216 to 230 us, 18-real), most
-// of them with smoother links (exp(0.15 i H): 410 to 560).
+// 2^64, infinities, NaN, or exponents near the ends of the range.  Where a site
+// falls back its warp pays both (24^3x48, us, every site in the chain / none:
+// 660 / 187 with 18-real links, 812 / 212 with 12; the chain alone took 537 and
+// 686).  On Gaussian fields no site does, on solutions and residuals of Gaussian
+// sources at most one warp in ten thousand (links of mean 0.94) holds one.  On
+// the propagator of a point source 0.1 to 2 % of the warps do (216 to 230 us,
+// 18-real), on residuals of such a solve most; smoother links have more
+// (propagators with exp(0.15 i H): 410 to 560 us).
 //
 // Instructions per hop: 30 conversions of 11 (a 64-bit shift written on two
 // 32-bit words: on a 64-bit variable the compiler took 16), 216 multiply-adds,
 // about 150 for the sums and their sizes and 60 for the scale.  The sizes and
 // the three bits that T has for the line at 2^-5 (a carry between the halves of
 // a row) cost 6 to 9 %: 174 -> 185 us and, with 12-real links, 193 -> 212 (the
-// links' own scale another 2 us with 18-real ones); at
-// 2^-3 without those bits the propagators above took the chain everywhere.
+// scale of 18-real links another 2); at 2^-3 without those bits the propagators
+// above took the chain everywhere.
 #pragma once
 
 #include <string.h>
