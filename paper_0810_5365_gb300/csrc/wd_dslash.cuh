@@ -585,9 +585,10 @@ __device__ __forceinline__ void hop_fix(FixSite& fx, int mu, const void* __restr
 // The eight hops of one FP64 site: fixed point, or the FP64 chain where the
 // values do not fit it.  24^3x48, one parity, us per launch: FP64 chain 537
 // (recon 18) and 686 (recon 12, which rebuilds row 2 on the FP64 pipe), fixed
-// point 187 and 212.  What bounds it now: the integer pipes (ALU 42 % busy)
-// through the latency of dependent instructions, with 12 warps per SM at 168
-// registers; 8 or 16 warps (255 registers, or 128 and spills) are slower.  The
+// point 187 and 212.  What bounds it now: the latency of dependent
+// integer instructions, with 12 warps per SM at 168 registers (12-real links:
+// integer multiply-adds 50 %, ALU 41 %, FP64 31 %, issue 42 %); 8 or 16 warps
+// (255 registers, or 128 and spills) are slower.  The
 // directions are a loop, not unrolled: eight copies of the hop (200 KB of
 // code) ran out of the instruction cache and took 500 us.
 template <int RC, bool DAG, bool COH>
